@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "pcc_internal.h"
+#include "pcc_totals.cuh"
 
 namespace pcc {
 
@@ -196,43 +197,18 @@ __global__ void commit_kernel(MRec sp, const int* __restrict__ cell_start, int* 
     cell_added[c] = 0;
 }
 
-// ---- FP64 totals: one warp per cell, fixed-order partials per block
-__global__ void totals_kernel(const pcc_species sp, int n_cells, int is_photon, double* __restrict__ partial)
+// ---- FP64 totals: slots shared out to the warps, fixed-order partials per block (see pcc_totals.cuh)
+template <bool PHOTON>
+__global__ void __launch_bounds__(256, 4) totals_kernel(const pcc_species sp, int n_cells, double* __restrict__ partial)
 {
-    __shared__ double acc[3][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int c = blockIdx.x * nw + wid; c < n_cells; c += gridDim.x * nw) {
-        const int b = sp.cell_start[c], n = sp.cell_count[c];
-        for (int k = lane; k < n; k += 32) {
-            const double ux = sp.ux[b + k], uy = sp.uy[b + k], uz = sp.uz[b + k], w = sp.w[b + k];
-            const double u = sqrt(ux * ux + uy * uy + uz * uz);
-            const double E = is_photon ? u : sqrt(1.0 + u * u);
-            s0 += w;
-            s1 += w * E;
-            s2 += w * u;
-        }
-    }
-    s0 = warp_sum(s0); s1 = warp_sum(s1); s2 = warp_sum(s2);
-    if (lane == 0) { acc[0][wid] = s0; acc[1][wid] = s1; acc[2][wid] = s2; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t0 = 0, t1 = 0, t2 = 0;
-        for (int k = 0; k < nw; ++k) { t0 += acc[0][k]; t1 += acc[1][k]; t2 += acc[2][k]; }
-        partial[3 * blockIdx.x + 0] = t0;
-        partial[3 * blockIdx.x + 1] = t1;
-        partial[3 * blockIdx.x + 2] = t2;
-    }
+    __shared__ double sh[3][32];
+    const int nw = blockDim.x >> 5;
+    TotalsAcc acc;
+    totals_share<PHOTON>(sp, n_cells, blockIdx.x * nw + (threadIdx.x >> 5), gridDim.x * nw, threadIdx.x & 31, acc);
+    totals_block_out(acc, sh, partial);
 }
 
-__global__ void totals_final_kernel(const double* partial, int nb, double* out)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double t0 = 0, t1 = 0, t2 = 0;
-        for (int b = 0; b < nb; ++b) { t0 += partial[3 * b]; t1 += partial[3 * b + 1]; t2 += partial[3 * b + 2]; }
-        out[0] = t0; out[1] = t1; out[2] = t2;
-    }
-}
+__global__ void totals_final_kernel(const double* partial, int nb, double* out) { totals_reduce(partial, nb, out); }
 
 }  // namespace pcc
 
@@ -340,13 +316,15 @@ extern "C" int pcc_totals(pcc_ctx* ctx, int n_cells, const pcc_species* sp, int 
                           void* stream)
 {
     if (!ctx || !sp || !out || n_cells < 1) { set_error("pcc_totals: invalid argument"); return PCC_E_INVALID; }
-    const int blocks = 2 * std::max(ctx->num_sms, 1);
+    // four resident blocks per SM, fewer where the cells do not fill them
+    const int blocks = std::min(4 * std::max(ctx->num_sms, 1), (n_cells + 7) / 8);
     int rc = ensure_scratch(ctx, (size_t)blocks * 3 * sizeof(double));
     if (rc) return rc;
     double* partial = (double*)ctx->scratch;
     cudaStream_t st = (cudaStream_t)stream;
-    totals_kernel<<<blocks, 256, 0, st>>>(*sp, n_cells, is_photon, partial);
-    totals_final_kernel<<<1, 32, 0, st>>>(partial, blocks, out);
+    if (is_photon) totals_kernel<true><<<blocks, 256, 0, st>>>(*sp, n_cells, partial);
+    else totals_kernel<false><<<blocks, 256, 0, st>>>(*sp, n_cells, partial);
+    totals_final_kernel<<<1, 96, 0, st>>>(partial, blocks, out);
     note_launches(2);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PCC_OK : cuda_fail(e, "pcc_totals");

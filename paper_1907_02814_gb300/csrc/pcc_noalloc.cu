@@ -25,11 +25,13 @@
 #include <string>
 
 #include "pcc_internal.h"
+#include "pcc_totals.cuh"
 
 namespace {
 
 constexpr int kCellsPerBlock = 1024;
 constexpr int kMaxBlocks = 4096;                       // at most 4,194,304 cells
+constexpr int kGridBlocks = 4 * 152;                   // four resident blocks on each SM
 constexpr long long kMaxCells = (long long)kCellsPerBlock * kMaxBlocks;
 
 // Per-block partial sums {sum W, sum W E, sum W |u|}; every block of a call
@@ -45,47 +47,20 @@ constexpr int kMaxContexts = 64;
 CachedAddress g_cache[kMaxContexts] = {};
 int g_cache_next = 0;
 
-// Block b sums the live particles of cells [b * 1024, (b + 1) * 1024), one warp
-// per cell at a time, lanes over particles; fixed-order reduction.
-__global__ void totals_block_kernel(const pcc_species sp, int n_cells, int is_photon, double* __restrict__ partial)
+// The slots of all cells shared out to the warps of the grid (see pcc_totals.cuh); fixed-order reduction.
+template <bool PHOTON>
+__global__ void __launch_bounds__(256, 4) totals_block_kernel(const pcc_species sp, int n_cells, double* __restrict__ partial)
 {
-    __shared__ double acc[3][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int c_begin = blockIdx.x * kCellsPerBlock;
-    const int c_end = min(c_begin + kCellsPerBlock, n_cells);
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int c = c_begin + wid; c < c_end; c += nw) {
-        const int b = sp.cell_start[c], n = sp.cell_count[c];
-        for (int k = lane; k < n; k += 32) {
-            const double ux = sp.ux[b + k], uy = sp.uy[b + k], uz = sp.uz[b + k], w = sp.w[b + k];
-            const double u = sqrt(ux * ux + uy * uy + uz * uz);
-            s0 += w;
-            s1 += w * (is_photon ? u : sqrt(1.0 + u * u));
-            s2 += w * u;
-        }
-    }
-    s0 = pcc::warp_sum(s0);
-    s1 = pcc::warp_sum(s1);
-    s2 = pcc::warp_sum(s2);
-    if (lane == 0) { acc[0][wid] = s0; acc[1][wid] = s1; acc[2][wid] = s2; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-        for (int k = 0; k < nw; ++k) { t0 += acc[0][k]; t1 += acc[1][k]; t2 += acc[2][k]; }
-        partial[3 * blockIdx.x + 0] = t0;
-        partial[3 * blockIdx.x + 1] = t1;
-        partial[3 * blockIdx.x + 2] = t2;
-    }
+    __shared__ double sh[3][32];
+    const int nw = blockDim.x >> 5;
+    pcc::TotalsAcc acc;
+    pcc::totals_share<PHOTON>(sp, n_cells, blockIdx.x * nw + (threadIdx.x >> 5), gridDim.x * nw, threadIdx.x & 31, acc);
+    pcc::totals_block_out(acc, sh, partial);
 }
 
 __global__ void totals_sum_kernel(const double* __restrict__ partial, int nb, double* __restrict__ out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-    for (int b = 0; b < nb; ++b) { t0 += partial[3 * b]; t1 += partial[3 * b + 1]; t2 += partial[3 * b + 2]; }
-    out[0] = t0;
-    out[1] = t1;
-    out[2] = t2;
+    pcc::totals_reduce(partial, nb, out);
 }
 
 // Identifier of the CUDA context current on this thread (cuCtxGetId; unique
@@ -169,10 +144,11 @@ extern "C" int pcc_totals_noalloc(int n_cells, const pcc_species* sp, int is_pho
     double* partial = nullptr;
     const int rc = partial_address(&partial);
     if (rc != PCC_OK) return rc;
-    const int nb = (n_cells + kCellsPerBlock - 1) / kCellsPerBlock;
+    const int nb = n_cells < 8 * kGridBlocks ? (n_cells + 7) / 8 : kGridBlocks;
     cudaStream_t st = (cudaStream_t)stream;
-    totals_block_kernel<<<nb, 256, 0, st>>>(*sp, n_cells, is_photon, partial);
-    totals_sum_kernel<<<1, 32, 0, st>>>(partial, nb, out);
+    if (is_photon) totals_block_kernel<true><<<nb, 256, 0, st>>>(*sp, n_cells, partial);
+    else totals_block_kernel<false><<<nb, 256, 0, st>>>(*sp, n_cells, partial);
+    totals_sum_kernel<<<1, 96, 0, st>>>(partial, nb, out);
     pcc::note_launches(2);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PCC_OK : pcc::cuda_fail(e, "pcc_totals_noalloc: launch");
