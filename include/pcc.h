@@ -254,7 +254,9 @@ int pcc_get_scan_classes(const pcc_ctx *ctx, int group, int *thresholds);
  * set PCC_ST_TIMEOUT and fall back to the global rows (same values), after
  * a second bounded wait that lets the copy land.  polls = 0 makes every
  * staged launch time out, to test the status path without a hang or a
- * fault.  Applies to later pcc_collide calls on this context; PCC_E_INVALID
+ * fault.  (A context with its own limit takes the launch sequence with the
+ * staged copies at every size; by default, calls of about 32 to 18000 cells
+ * run as one kernel without them, with the same results.)  Applies to later pcc_collide calls on this context; PCC_E_INVALID
  * for polls < 0. */
 int pcc_set_wait_limit(pcc_ctx *ctx, int polls);
 

@@ -4,6 +4,7 @@
 #include <cmath>
 #include <vector>
 
+#include "pcc_commit.cuh"
 #include "pcc_internal.h"
 #include "pcc_totals.cuh"
 
@@ -167,34 +168,10 @@ __global__ void cell_sort_kernel(const int* __restrict__ cell_start, const int* 
 }
 
 // ---- commit of appended secondaries: order by pid, then make live
-__global__ void commit_kernel(MRec sp, const int* __restrict__ cell_start, int* __restrict__ cell_count,
-                              int* __restrict__ cell_added, int n_cells)
+__global__ void commit_kernel(SpeciesView sp, int n_cells)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_cells) return;
-    const int a = cell_added[c];
-    if (a == 0) return;
-    const int b = cell_start[c] + cell_count[c];
-    for (int i = 1; i < a; ++i) {   // insertion sort of the (few) appended records
-        const uint64_t kp = sp.pid[b + i];
-        const float vx = sp.ux[b + i], vy = sp.uy[b + i], vz = sp.uz[b + i], vw = sp.w[b + i];
-        const float vxx = sp.x ? sp.x[b + i] : 0.f;
-        int j = i - 1;
-        while (j >= 0 && sp.pid[b + j] > kp) {
-            sp.pid[b + j + 1] = sp.pid[b + j];
-            sp.ux[b + j + 1] = sp.ux[b + j];
-            sp.uy[b + j + 1] = sp.uy[b + j];
-            sp.uz[b + j + 1] = sp.uz[b + j];
-            sp.w[b + j + 1] = sp.w[b + j];
-            if (sp.x) sp.x[b + j + 1] = sp.x[b + j];
-            --j;
-        }
-        sp.pid[b + j + 1] = kp;
-        sp.ux[b + j + 1] = vx; sp.uy[b + j + 1] = vy; sp.uz[b + j + 1] = vz; sp.w[b + j + 1] = vw;
-        if (sp.x) sp.x[b + j + 1] = vxx;
-    }
-    cell_count[c] += a;
-    cell_added[c] = 0;
+    if (c < n_cells) commit_cell(sp, c);
 }
 
 // ---- FP64 totals: slots shared out to the warps, fixed-order partials per block (see pcc_totals.cuh)
@@ -304,9 +281,7 @@ extern "C" int pcc_append_secondaries(pcc_ctx* ctx, int n_cells, pcc_species* sp
         set_error("pcc_append_secondaries: invalid argument");
         return PCC_E_INVALID;
     }
-    MRec r{sp->ux, sp->uy, sp->uz, sp->w, sp->x, sp->pid};
-    commit_kernel<<<(n_cells + 255) / 256, 256, 0, (cudaStream_t)stream>>>(r, sp->cell_start, sp->cell_count,
-                                                                            sp->cell_added, n_cells);
+    commit_kernel<<<(n_cells + 255) / 256, 256, 0, (cudaStream_t)stream>>>(view_of(*sp), n_cells);
     note_launches(1);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PCC_OK : cuda_fail(e, "pcc_append_secondaries");

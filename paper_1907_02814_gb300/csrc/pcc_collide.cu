@@ -8,23 +8,11 @@
 //                   copy (cp.async.bulk + mbarrier).
 #include <algorithm>
 
+#include "pcc_commit.cuh"
 #include "pcc_internal.h"
 #include "pcc_physics.cuh"
 
 namespace pcc {
-
-struct SpeciesView {
-    float *ux, *uy, *uz, *w, *x;
-    uint64_t* pid;
-    const int* start;
-    int* count;
-    int* added;
-};
-
-__host__ __device__ inline SpeciesView view_of(const pcc_species& s)
-{
-    return SpeciesView{s.ux, s.uy, s.uz, s.w, s.x, s.pid, s.cell_start, s.cell_count, s.cell_added};
-}
 
 struct StepArgs {
     int n_cells;
@@ -798,6 +786,18 @@ struct CellList {
                      // [thr[2], thr[1]) 8, [thr[3], thr[2]) 4, below 2 (pcc_set_scan_classes)
 };
 
+// Calls of kFusedMinCells cells up to kFusedCellsPerWarp for each resident warp
+// (24 on an SM: 18240 cells on 152 SMs) run as one kernel, a warp per cell (see
+// fused_cell_kernel).  Step in a graph, one kernel against the general sequence:
+// 64 cells 10-18 against 87-102 us; 16384 cells of 64 to 256 electrons 47-75
+// against 103-118 us, log-normal ones 65-89 against 120-136 us; at 32768 cells
+// 84-152 against 109-148 us and for log-normal ones 122-179 against 131-165 us,
+// since the large cells, which the general scan takes first, hold up a warp.
+// (Log-normal cells with as many ions as electrons in a step so long that large
+// cells collide on most pairs are the exception: 490 against 280 us at 16384.)
+constexpr int kFusedMinCells = 32;
+constexpr int kFusedCellsPerWarp = 5;
+constexpr int kFusedWarpsPerSM = 24;
 constexpr int kClassBlock = 1024;                 // cells per class-sort block
 constexpr int kClassSmemMax = 200 * 1024;         // offsets scanned in shared memory up to this size
 
@@ -1254,6 +1254,13 @@ __device__ __forceinline__ T group_sum(T v)
 {
 #pragma unroll
     for (int o = G >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+__device__ __forceinline__ float warp_max(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
 
@@ -1720,6 +1727,83 @@ __device__ __forceinline__ void fold_acc(Acc& acc, BlockAcc& bacc, DevStats* st)
     block_acc_flush(bacc, st);
 }
 
+// Evaluates pair j (projectile slot s, target t, pass m) of a cell whose accept
+// digits passed the quick reject: ion frame, cross section, acceptance and
+// event; true when the projectile changed.  PH: photons, else group (e- or e+).
+template <bool PH>
+__device__ __forceinline__ bool eval_pair(const StepArgs& a, const Tab<float>& tb, int group, int cell, const CellRec& cm,
+                                          uint32_t s, uint32_t j, uint32_t t, uint32_t m, Acc& acc, float& rad, float& wcre)
+{
+    const SpeciesView& P = PH ? a.ph : (group == kGroupEm ? a.em : a.ep);
+    using AS = AcceptSlots<PH ? kGroupPh : kGroupEm>;
+    const uint32_t dg = AS::digit(s);
+    const Philox4 ph = draw_k(AS::ctr(s), (uint32_t)cell, (uint32_t)a.step, stream_tag(group, kAccept, m), a.keys);
+    const uint32_t r1 = accept_digit(ph, dg), r2 = PH ? 0u : accept_digit(ph, dg + 1);
+    const AcceptSrc src{AS::ext(s), (uint32_t)cell, stream_tag(group, kAcceptExt, m)};
+    const int ts = cm.t0 + (int)t, sl = cm.p0 + (int)s;
+    if (PH) return bh_candidate(a, tb, cell, cm.mat, cm.coef, sl, ts, j, r1, src, acc, wcre);
+    bool event = false;
+    float u[3] = {P.ux[sl], P.uy[sl], P.uz[sl]};
+    const float xp = P.x ? P.x[sl] : 0.f;
+    ei_pair<float>(&a, tb, group, cell, cm.mat, a.f_Z[cm.mat], cm.coef, u, P.w + sl, xp, ts, j, r1, r2, src, acc, rad, wcre,
+                   event);
+    if (event) {
+        P.ux[sl] = u[0]; P.uy[sl] = u[1]; P.uz[sl] = u[2];
+    }
+    return event;
+}
+
+__device__ __forceinline__ PermKeys perm_keys(const StepArgs& a, int group, int cell)
+{
+    const Philox4 kp = draw_k(0, (uint32_t)cell, (uint32_t)a.step, stream_tag(group, kPerm, 0), a.keys);
+    return PermKeys{{kp.v[0], kp.v[1], kp.v[2], kp.v[3]}};
+}
+
+// A candidate of a cell with N_p >= N_t (one pair per projectile slot s).
+template <bool PH>
+__device__ __forceinline__ bool flat_pair(const StepArgs& a, const Tab<float>& tb, int group, int cell, const CellRec& cm,
+                                          uint32_t s, Acc& acc, float& rad, float& wcre)
+{
+    const PermKeys rk = perm_keys(a, group, cell);
+    const uint32_t j = cm.Np <= 32 ? perm_pos_small(s, cm.Np, rk) : perm_pos_large(s, cm.Np, rk);
+    return eval_pair<PH>(a, tb, group, cell, cm, s, j, fast_mod(j, cm.Nt, 1.0f / (float)cm.Nt), 0u, acc, rad, wcre);
+}
+
+// The cnt candidates (pair indices qb, increasing for each projectile) of a
+// cell with N_p < N_t, by all 32 lanes: a lane per candidate, and candidates of
+// the same projectile among them one after the other, since its momentum after
+// one event enters the next and an absorbed photon skips its later pairs.  (On
+// one lane the list of a large cell was the longest chain of the call.)  tab:
+// 32 ints for the P table of short lists.  True when the lane changed a projectile.
+template <bool PH>
+__device__ __forceinline__ bool caseb_pairs(const StepArgs& a, const Tab<float>& tb, int group, int cell, const CellRec& cm,
+                                            const uint32_t* qb, int cnt, int* tab, int lane, Acc& acc, float& rad,
+                                            float& wcre)
+{
+    const uint32_t Np = cm.Np, Nt = cm.Nt;
+    const PermKeys rk = perm_keys(a, group, cell);
+    __syncwarp();
+    if (Nt <= 32 && lane < (int)Nt) tab[perm_pos_small(lane, Nt, rk)] = lane;   // P table of the targets
+    __syncwarp();
+    bool any = false;
+    for (int k0 = 0; k0 < cnt; k0 += 32) {
+        const bool valid = k0 + lane < cnt;
+        const uint32_t j = valid ? qb[k0 + lane] : 0u;
+        const uint32_t m = j / Np, s = j - m * Np;
+        const unsigned peers = __match_any_sync(0xffffffffu, valid ? s : 0x80000000u | (uint32_t)lane);
+        const int turn = __popc(peers & ((1u << lane) - 1u));
+        const int turns = __reduce_max_sync(0xffffffffu, turn);
+        for (int r = 0; r <= turns; ++r) {
+            if (valid && turn == r && !(PH && a.ph.w[cm.p0 + (int)s] == 0.f)) {
+                const uint32_t t = Nt <= 32 ? (uint32_t)tab[j] : perm_elem_large(j, Nt, rk);
+                any |= eval_pair<PH>(a, tb, group, cell, cm, s, j, t, m, acc, rad, wcre);
+            }
+            __syncwarp();
+        }
+    }
+    return any;
+}
+
 // Candidates of cells with N_p >= N_t (one pair per projectile), one thread
 // each: pairing, ion frame, cross section, acceptance, events.  Event
 // contributions to the cell ledger are gathered per cell (float atomics) and
@@ -1737,8 +1821,6 @@ __global__ void __launch_bounds__(kBatchedThreads, 4) flat_cand_kernel(const __g
     if (st0 && threadIdx.x == 0) bacc.status |= st0;
     __syncthreads();
     const Tab<float> tb = batched_tab<GROUP>(a, ls);
-    const SpeciesView& P = GROUP == kGroupEm ? a.em : (GROUP == kGroupEp ? a.ep : a.ph);
-    const uint32_t step32 = (uint32_t)a.step;
     const int total = min(*Q.flat_count, (int)Q.cap_flat);
     Acc acc;
     acc.zero();
@@ -1748,32 +1830,8 @@ __global__ void __launch_bounds__(kBatchedThreads, 4) flat_cand_kernel(const __g
         const uint32_t s = e.y;
         if (cell < 0 || cell >= a.n_cells) continue;
         const CellRec cm = load_rec(Q, cell);
-        const uint32_t Np = cm.Np, Nt = cm.Nt;
-        const float coef = cm.coef;
-        const Philox4 kp = draw_k(0, (uint32_t)cell, step32, stream_tag(GROUP, kPerm, 0), a.keys);
-        PermKeys rk;
-        rk.k[0] = kp.v[0]; rk.k[1] = kp.v[1]; rk.k[2] = kp.v[2]; rk.k[3] = kp.v[3];
-        const uint32_t j = Np <= 32 ? perm_pos_small(s, Np, rk) : perm_pos_large(s, Np, rk);
-        const int ts = cm.t0 + (int)fast_mod(j, Nt, 1.0f / (float)Nt);
-        using AS = AcceptSlots<GROUP>;
-        const uint32_t dg = AS::digit(s);
-        const Philox4 ph = draw_k(AS::ctr(s), (uint32_t)cell, step32, stream_tag(GROUP, kAccept, 0), a.keys);
-        const uint32_t r1 = accept_digit(ph, dg), r2 = GROUP == kGroupPh ? 0u : accept_digit(ph, dg + 1);
-        const AcceptSrc src{AS::ext(s), (uint32_t)cell, stream_tag(GROUP, kAcceptExt, 0)};
-        const int sl = cm.p0 + (int)s;
         float rad = 0.f, wcre = 0.f;
-        bool event = false;
-        if (GROUP == kGroupPh) {
-            event = bh_candidate(a, tb, cell, cm.mat, coef, sl, ts, j, r1, src, acc, wcre);
-        } else {
-            float u[3] = {P.ux[sl], P.uy[sl], P.uz[sl]};
-            const float xp = P.x ? P.x[sl] : 0.f;
-            ei_pair<float>(&a, tb, GROUP, cell, cm.mat, a.f_Z[cm.mat], coef, u, P.w + sl, xp, ts, j, r1, r2, src, acc,
-                           rad, wcre, event);
-            if (event) {
-                P.ux[sl] = u[0]; P.uy[sl] = u[1]; P.uz[sl] = u[2];
-            }
-        }
+        const bool event = flat_pair<GROUP == kGroupPh>(a, tb, GROUP, cell, cm, s, acc, rad, wcre);
         if (event) {
             if (rad != 0.f) atomicAdd(&Q.evacc[cell].x, rad);
             if (wcre != 0.f) atomicAdd(&Q.evacc[cell].y, wcre);
@@ -1783,9 +1841,7 @@ __global__ void __launch_bounds__(kBatchedThreads, 4) flat_cand_kernel(const __g
     fold_acc(acc, bacc, a.st);
 }
 
-// Candidates of cells with N_p < N_t, one warp per cell, in queue order on
-// one lane (a projectile's pairs in increasing pair index; a photon absorbed
-// on an earlier pair skips its later ones).
+// Candidates of cells with N_p < N_t, one warp per cell (see caseb_pairs).
 template <int GROUP>
 __global__ void __launch_bounds__(kBatchedThreads, 2) caseb_cand_kernel(const __grid_constant__ StepArgs a, Queue Q,
                                                                         int stage_bytes)
@@ -1804,58 +1860,17 @@ __global__ void __launch_bounds__(kBatchedThreads, 2) caseb_cand_kernel(const __
     int* tab = scratch[wid];
     const int n = *Q.caseb_count;
     const int nwarps = gridDim.x * (blockDim.x >> 5);
-    const SpeciesView& P = GROUP == kGroupEm ? a.em : (GROUP == kGroupEp ? a.ep : a.ph);
-    const uint32_t step32 = (uint32_t)a.step;
     Acc acc;
     acc.zero();
     for (int kk = blockIdx.x * (blockDim.x >> 5) + wid; kk < n; kk += nwarps) {
         const int cell = Q.caseb[kk];
         if (cell < 0 || cell >= a.n_cells) continue;
         const CellRec cm = load_rec(Q, cell);
-        const uint32_t Np = cm.Np, Nt = cm.Nt;
-        const int cnt = Q.cand[cell];
-        const float coef = cm.coef;
-        const Philox4 kp = draw_k(0, (uint32_t)cell, step32, stream_tag(GROUP, kPerm, 0), a.keys);
-        PermKeys rk;
-        rk.k[0] = kp.v[0]; rk.k[1] = kp.v[1]; rk.k[2] = kp.v[2]; rk.k[3] = kp.v[3];
-        if (Nt <= 32) {   // P table of the targets
-            __syncwarp();
-            if (lane < (int)Nt) tab[perm_pos_small(lane, Nt, rk)] = lane;
-            __syncwarp();
-        }
-        if (lane == 0) {
-            float rad = 0.f, wcre = 0.f;
-            bool any = false;
-            for (int k = 0; k < cnt; ++k) {
-                const uint32_t j = Q.qb[cm.t0 + k];
-                const uint32_t s = j % Np, mp = j / Np;
-                using AS = AcceptSlots<GROUP>;
-                const uint32_t dg = AS::digit(s);
-                const Philox4 ph = draw_k(AS::ctr(s), (uint32_t)cell, step32, stream_tag(GROUP, kAccept, mp), a.keys);
-                const uint32_t r1 = accept_digit(ph, dg), r2 = GROUP == kGroupPh ? 0u : accept_digit(ph, dg + 1);
-                const AcceptSrc src{AS::ext(s), (uint32_t)cell, stream_tag(GROUP, kAcceptExt, mp)};
-                const uint32_t t = Nt <= 32 ? (uint32_t)tab[j] : perm_elem_large(j, Nt, rk);
-                const int ts = cm.t0 + (int)t, sl = cm.p0 + (int)s;
-                bool event = false;
-                if (GROUP == kGroupPh) {
-                    if (P.w[sl] == 0.f) continue;   // absorbed earlier in this step
-                    event = bh_candidate(a, tb, cell, cm.mat, coef, sl, ts, j, r1, src, acc, wcre);
-                } else {
-                    float u[3] = {P.ux[sl], P.uy[sl], P.uz[sl]};
-                    const float xp = P.x ? P.x[sl] : 0.f;
-                    ei_pair<float>(&a, tb, GROUP, cell, cm.mat, a.f_Z[cm.mat], coef, u, P.w + sl, xp, ts, j, r1, r2,
-                                   src, acc, rad, wcre, event);
-                    if (event) {
-                        P.ux[sl] = u[0]; P.uy[sl] = u[1]; P.uz[sl] = u[2];
-                    }
-                }
-                any |= event;
-            }
-            if (any) {
-                if (rad != 0.f) atomicAdd(&Q.evacc[cell].x, rad);
-                if (wcre != 0.f) atomicAdd(&Q.evacc[cell].y, wcre);
-                flag_cell(Q, cell);
-            }
+        float rad = 0.f, wcre = 0.f;
+        if (caseb_pairs<GROUP == kGroupPh>(a, tb, GROUP, cell, cm, Q.qb + cm.t0, Q.cand[cell], tab, lane, acc, rad, wcre)) {
+            if (rad != 0.f) atomicAdd(&Q.evacc[cell].x, rad);
+            if (wcre != 0.f) atomicAdd(&Q.evacc[cell].y, wcre);
+            flag_cell(Q, cell);
         }
         __syncwarp();
     }
@@ -1967,6 +1982,400 @@ __global__ void finalize_kernel(const __grid_constant__ StepArgs a, Queue Q)
         __syncwarp();
         if (lane == 0) Q.flag[cell] = 0;
     }
+}
+
+// ---- a whole step per cell -------------------------------------------------------
+// One warp takes a cell through all three groups: sums, accept digits,
+// candidates, events, ledger, removal of absorbed photons and, for the steps of
+// a graph, the commit of the secondaries.  Nothing is sorted, zeroed or queued
+// between kernels, so a step is one launch instead of the fifteen of the
+// general sequence (and three commits), each a few microseconds of fill and
+// drain: that is what bounds calls of up to some ten thousand cells.  The FP32
+// sums are taken by the lane group (of 2 to 32 lanes) that the general scan
+// would give the cell, in its order, so the coefficient and every decision are
+// the same bits on both paths.  A warp scans up to kFusedBatch cells, all groups
+// (no group's sums or digits depend on another group's events), and evaluates
+// the candidates of all of them together: one at a time, they would leave most
+// lanes idle through its long chain of dependent loads.
+struct FusedArgs {
+    int thr[3][4];      // scan lane groups per group (see CellList)
+    unsigned run;       // bit g: group g takes part
+    uint32_t* qb;       // [target capacity] pair indices of candidates in cells with N_p < N_t
+};
+
+constexpr int kFusedWarps = kBatchedThreads / 32;
+constexpr int kFusedBatch = 8;      // cells scanned before their candidates are evaluated
+constexpr int kFusedQueue = 1024;   // staged candidates: all that one pass of the accept loop can mark
+
+struct FusedWarp {
+    float2 ev[kFusedBatch][3];      // radiated energy and created weight of the cell's events
+    struct { int p0; uint32_t Np; float coef; int cnt_b; } rec[kFusedBatch][3];   // cnt_b: candidates if N_p < N_t
+    struct { int cell, t0, mat; uint32_t Nt; } cell[kFusedBatch];
+    unsigned changed;               // bit 4b + g: an event in group g of cell b
+    int tab[64];
+    uint32_t q[kFusedQueue];        // slot << 5 | b << 2 | g
+};
+
+__device__ __forceinline__ CellRec fused_rec(const FusedWarp& w, int b, int g)
+{
+    CellRec c;
+    c.p0 = w.rec[b][g].p0; c.Np = w.rec[b][g].Np; c.coef = w.rec[b][g].coef;
+    c.t0 = w.cell[b].t0; c.Nt = w.cell[b].Nt; c.mat = w.cell[b].mat;
+    return c;
+}
+
+// A thread's counters to the block's.
+__device__ __forceinline__ void add_rare(const Acc& acc, BlockAcc& b)
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        if (acc.accepted[i]) atomicAdd(&b.accepted[i], (unsigned long long)acc.accepted[i]);
+        if (acc.created[i]) atomicAdd(&b.created[i], (unsigned long long)acc.created[i]);
+    }
+    if (acc.dE != 0.0) atomicAdd(&b.dE, acc.dE);
+    if (acc.status) atomicOr(&b.status, acc.status);
+}
+
+__device__ __forceinline__ void fused_event(FusedWarp& w, int b, int g, float rad, float wcre)
+{
+    if (rad != 0.f) atomicAdd(&w.ev[b][g].x, rad);
+    if (wcre != 0.f) atomicAdd(&w.ev[b][g].y, wcre);
+    atomicOr(&w.changed, 1u << (4 * b + g));
+}
+
+__device__ __forceinline__ void fused_candidate(const StepArgs& a, FusedWarp& w, uint32_t e, Acc& acc)
+{
+    const Tab<float> tb{a.f_brems_lnsig, a.f_brems_cdf, a.f_bh_lnsig, a.f_bh_cdf, a.f_tri_gp, a.f_tri_split};
+    const uint32_t s = e >> 5;
+    const int b = (int)(e >> 2) & 7, g = (int)(e & 3u), cell = w.cell[b].cell;
+    const CellRec cm = fused_rec(w, b, g);
+    float rad = 0.f, wcre = 0.f;
+    const bool event = g == kGroupPh ? flat_pair<true>(a, tb, g, cell, cm, s, acc, rad, wcre)
+                                     : flat_pair<false>(a, tb, g, cell, cm, s, acc, rad, wcre);
+    if (event) fused_event(w, b, g, rad, wcre);
+}
+
+// The staged candidates of one warp (when its list is full), or of all warps
+// of the block together, so that a cell full of candidates does not hold
+// up one warp.  Out of line, as the other rare paths, so that the scan of the
+// mostly candidate-free cells keeps its registers (inlined, the kernel spilled
+// 734 bytes).
+__device__ __noinline__ void fused_drain(const StepArgs* ap, FusedWarp* w, int nq, BlockAcc* bacc)
+{
+    __syncwarp();
+    Acc acc;
+    acc.zero();
+    for (int i = threadIdx.x & 31; i < nq; i += 32) fused_candidate(*ap, *w, w->q[i], acc);
+    add_rare(acc, *bacc);
+    __syncwarp();
+}
+
+__device__ __noinline__ void fused_drain_block(const StepArgs* ap, FusedWarp* work, const int* staged, BlockAcc* bacc)
+{
+    int total = 0;
+#pragma unroll
+    for (int k = 0; k < kFusedWarps; ++k) total += staged[k];
+    if (threadIdx.x >= total) return;
+    Acc acc;
+    acc.zero();
+    for (int i = threadIdx.x; i < total; i += kBatchedThreads) {
+        int k = 0, r = i;
+        while (r >= staged[k]) r -= staged[k++];
+        fused_candidate(*ap, work[k], work[k].q[r], acc);
+    }
+    add_rare(acc, *bacc);
+}
+
+// The queued candidates of cell b's group g with N_p < N_t.  All 32 lanes.
+__device__ __noinline__ void fused_caseb(const StepArgs* ap, const uint32_t* qb, FusedWarp* w, int b, int g, BlockAcc* bacc)
+{
+    const StepArgs& a = *ap;
+    const Tab<float> tb{a.f_brems_lnsig, a.f_brems_cdf, a.f_bh_lnsig, a.f_bh_cdf, a.f_tri_gp, a.f_tri_split};
+    const int lane = threadIdx.x & 31, cell = w->cell[b].cell, cnt = w->rec[b][g].cnt_b;
+    const CellRec cm = fused_rec(*w, b, g);
+    Acc acc;
+    acc.zero();
+    float rad = 0.f, wcre = 0.f;
+    const bool event = g == kGroupPh ? caseb_pairs<true>(a, tb, g, cell, cm, qb + cm.t0, cnt, w->tab, lane, acc, rad, wcre)
+                                     : caseb_pairs<false>(a, tb, g, cell, cm, qb + cm.t0, cnt, w->tab, lane, acc, rad, wcre);
+    if (event) fused_event(*w, b, g, rad, wcre);
+    add_rare(acc, *bacc);
+    __syncwarp();
+}
+
+// Cell b's ledger (the groups in order) and the removal of its absorbed photons.
+__device__ __noinline__ void fused_finish(const StepArgs* ap, FusedWarp* w, int b)
+{
+    const StepArgs& a = *ap;
+    const int lane = threadIdx.x & 31, cell = w->cell[b].cell;
+    const unsigned ch = w->changed >> (4 * b);
+    if (lane == 0 && a.ledger) {
+        float4* Lg = reinterpret_cast<float4*>(a.ledger) + cell;
+        const float4 v = *Lg;
+        Kahan ka{v.x, v.y}, kb{v.z, v.w};
+        for (int g = 0; g < 3; ++g) {
+            if (!(ch >> g & 1u)) continue;
+            ka.add(w->ev[b][g].x);
+            kb.add(w->ev[b][g].y);
+        }
+        *Lg = make_float4(ka.s, ka.c, kb.s, kb.c);
+    }
+    __syncwarp();
+    if (ch >> kGroupPh & 1u) compact_region_warp(a.ph, cell);
+    __syncwarp();
+}
+
+__device__ __noinline__ void fused_commit(const StepArgs* a, int species, int cell)
+{
+    if (species == 0) commit_cell(a->em, cell);
+    else if (species == 1) commit_cell(a->ep, cell);
+    else commit_cell(a->ph, cell);
+}
+
+__device__ __noinline__ float fused_npt(const StepArgs* a, int group, int cell, int p0, int t0, uint32_t Np, uint32_t Nt,
+                                        int* tab, int lane)
+{
+    if (group == kGroupEm) return npt_over_pairs<kGroupEm>(*a, a->em, cell, p0, t0, Np, Nt, tab, lane);
+    if (group == kGroupEp) return npt_over_pairs<kGroupEp>(*a, a->ep, cell, p0, t0, Np, Nt, tab, lane);
+    return npt_over_pairs<kGroupPh>(*a, a->ph, cell, p0, t0, Np, Nt, tab, lane);
+}
+
+// Sum over the first G lanes (the others hold 0) as group_sum<G> takes it, on every lane.
+__device__ __forceinline__ float lanes_sum(float v, int G)
+{
+#pragma unroll 1
+    for (int o = G >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return __shfl_sync(0xffffffffu, v, 0);
+}
+
+// What the electron group leaves of the cell's ions for the other two (see IonCache).
+struct IonSums {
+    bool have;
+    float n_t, w0, fac;
+    bool uni;
+};
+
+// Scan of one group of cell b of the batch: sums, coefficient, accept digits;
+// candidates staged in w.q (nq of them so far) or, with N_p < N_t, in F.qb.
+template <int GROUP>
+__device__ __forceinline__ void fused_scan(const StepArgs& a, const FusedArgs& F, FusedWarp& w, int b, int cell, int p0,
+                                           uint32_t Np, int t0, uint32_t Nt, int mat, IonSums& is, int& nq, int lane,
+                                           BlockAcc& bacc)
+{
+    constexpr unsigned kFull = 0xffffffffu;
+    const SpeciesView& P = GROUP == kGroupEm ? a.em : (GROUP == kGroupEp ? a.ep : a.ph);
+    const SpeciesView& I = a.ion;
+    const uint32_t step32 = (uint32_t)a.step;
+    const bool caseA = Np >= Nt;
+    const int cls = size_class((int)Np, (int)Nt);
+    const int* thr = F.thr[GROUP];
+    const int G = cls >= thr[0] ? 32 : cls >= thr[1] ? 16 : cls >= thr[2] ? 8 : cls >= thr[3] ? 4 : 2;
+    const uint32_t l0 = lane < G ? (uint32_t)lane : 0x40000000u;   // lanes past the group sum nothing
+    // ---- sums, as in scan_segment
+    if (GROUP == kGroupEm || !is.have) {
+        const float w0 = I.w[t0];
+        float st = 0.f, u2m = 0.f, u2s = 0.f;
+        bool uni = true;
+#pragma unroll 4
+        for (uint32_t s = l0; s < Nt; s += G) {
+            const float wt = I.w[t0 + s];
+            st += wt;
+            uni &= (wt == w0);
+            if constexpr (GROUP == kGroupEm) {
+                const float ux = I.ux[t0 + s], uy = I.uy[t0 + s], uz = I.uz[t0 + s];
+                const float u2 = ux * ux + uy * uy + uz * uz;
+                u2m = fmaxf(u2m, u2);
+                u2s += u2;
+            }
+        }
+        is.n_t = lanes_sum(st, G);
+        is.w0 = w0;
+        is.uni = __all_sync(kFull, uni);
+        if constexpr (GROUP == kGroupEm) {
+            const float bm = fminf(warp_max(isfinite(u2s) && u2m < 1e30f ? __fdividef(u2m, 1.f + u2m) : 1.f), 1.f);
+            is.fac = fminf((1.f + (bm > 0.f ? bm * rsqrtf(bm) : 0.f)) * (1.f + 0x1p-20f), 2.f);
+            is.have = true;
+        } else {
+            is.fac = 2.f;
+        }
+    }
+    float sp = 0.f, sf = 0.f;
+    const float w0 = is.w0;
+    if (caseA) {
+        const uint32_t al = (uint32_t)((reinterpret_cast<uintptr_t>(P.w + p0) >> 2) & 3u);
+        const uint32_t hd = min((4u - al) & 3u, Np), nb = (Np - hd) >> 2, tl = Np - hd - 4 * nb;
+        const float4* W4 = reinterpret_cast<const float4*>(P.w + p0 + hd);
+#pragma unroll 2
+        for (uint32_t v = l0; v < nb; v += G) {
+            const float4 q = W4[v];
+            sp += (q.x + q.y) + (q.z + q.w);
+            sf += (fminf(q.x, w0) + fminf(q.y, w0)) + (fminf(q.z, w0) + fminf(q.w, w0));
+        }
+#pragma unroll 1
+        for (uint32_t i = l0; i < hd + tl; i += G) {
+            const float wp = P.w[p0 + (i < hd ? i : 4 * nb + i)];
+            sp += wp;
+            sf += fminf(wp, w0);
+        }
+    } else {
+        const uint32_t q0 = Nt / Np, r0 = Nt - q0 * Np;
+#pragma unroll 1
+        for (uint32_t s = l0; s < Np; s += G) {
+            const float wp = P.w[p0 + s];
+            sp += wp;
+            sf += fminf(wp, w0) * (float)(q0 + (s < r0 ? 1u : 0u));
+        }
+    }
+    const float n_p = lanes_sum(sp, G);
+    const float n_pt = is.uni ? lanes_sum(sf, G) : fused_npt(&a, GROUP, cell, p0, t0, Np, Nt, w.tab, lane);
+    const float coef = __fdividef(n_p, n_pt) * is.n_t * a.f_cdt;
+    uint32_t k1, k2;
+    bound_thresholds<GROUP>(a, mat, coef * (0.5f * is.fac), k1, k2);
+    if (lane == 0) {
+        w.rec[b][GROUP].p0 = p0; w.rec[b][GROUP].Np = Np; w.rec[b][GROUP].coef = coef;
+        atomicAdd(&bacc.pairs[GROUP], (unsigned long long)(caseA ? Np : Nt));
+        if ((caseA ? Np : Nt) > 65536u || (uint32_t)cell > 0xFFFFFFu || a.step > 0x7FFFFull)
+            atomicOr(&bacc.status, PCC_ST_ID_RANGE);
+    }
+    // ---- accept digits and candidates
+    using AS = AcceptSlots<GROUP>;
+    constexpr uint32_t S = AS::kPerDraw;
+    if (caseA) {
+        constexpr uint32_t kIt = 32 / S;   // iterations per candidate mask
+        const uint32_t nit = (Np + S * 32 - 1) / (S * 32);
+        const PhiloxFixed pf = philox_fixed((uint32_t)cell, step32, stream_tag(GROUP, kAccept, 0), a.keys);
+#pragma unroll 1
+        for (uint32_t it0 = 0; it0 < nit; it0 += kIt) {
+            const uint32_t ite = min(it0 + kIt, nit);
+            uint32_t cmask = 0;
+#pragma unroll 1
+            for (uint32_t it = it0; it < ite; ++it) {
+                const Philox4 ph = draw_fixed(it * 32 + lane, pf, a.keys);
+                const uint32_t s0 = (it * 32 + lane) * S, lim = s0 < Np ? Np - s0 : 0u;
+#pragma unroll
+                for (int h = 0; h < (int)S; ++h)
+                    if ((uint32_t)h < lim && AS::hit(ph, h, k1, k2)) cmask |= 1u << ((it - it0) * S + h);
+            }
+            if (!__any_sync(kFull, cmask != 0u)) continue;
+            const uint32_t n = __popc(cmask);
+            uint32_t incl = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const int total = (int)__shfl_sync(kFull, incl, 31);
+            if (lane == 0) atomicAdd(&bacc.candidates[GROUP], (unsigned long long)total);
+            if (nq + total > kFusedQueue) {
+                fused_drain(&a, &w, nq, &bacc);
+                nq = 0;
+            }
+            uint32_t k = (uint32_t)nq + incl - n;
+#pragma unroll 1
+            while (cmask) {
+                const uint32_t c = (uint32_t)(__ffs(cmask) - 1);
+                cmask &= cmask - 1u;
+                w.q[k++] = (((it0 + c / S) * 32 + (uint32_t)lane) * S + c % S) << 5 | (uint32_t)b << 2 | (uint32_t)GROUP;
+            }
+            nq += total;
+        }
+    } else {
+        const unsigned below = (1u << lane) - 1u;
+        const uint32_t Qn = (Np + S - 1) / S, units = Qn * ((Nt + Np - 1) / Np);
+        const float inv_qn = 1.0f / (float)Qn;
+        uint32_t cnt = 0;
+#pragma unroll 1
+        for (uint32_t i0 = 0; i0 < units; i0 += 32) {
+            const uint32_t i = i0 + lane;
+            const bool valid = i < units;
+            uint32_t mp = 0u, q = 0u;
+            if (valid) div_small(i, Qn, inv_qn, mp, q);
+            const Philox4 ph = draw_k(q, (uint32_t)cell, step32, stream_tag(GROUP, kAccept, mp), a.keys);
+            bool c[S], anyc = false;
+#pragma unroll
+            for (int h = 0; h < (int)S; ++h) {
+                const uint32_t s = S * q + h;
+                c[h] = valid && s < Np && s + mp * Np < Nt && AS::hit(ph, h, k1, k2);
+                anyc |= c[h];
+            }
+            if (!__any_sync(kFull, anyc)) continue;
+#pragma unroll
+            for (int h = 0; h < (int)S; ++h) {
+                const unsigned m = __ballot_sync(kFull, c[h]);
+                if (c[h]) F.qb[t0 + cnt + __popc(m & below)] = S * q + h + mp * Np;
+                cnt += __popc(m);
+            }
+        }
+        if (cnt) {   // warp-uniform
+            // the three groups share the cell's part of qb, so its list is worked off now
+            if (lane == 0) {
+                atomicAdd(&bacc.candidates[GROUP], (unsigned long long)cnt);
+                w.rec[b][GROUP].cnt_b = (int)cnt;
+            }
+            __syncwarp();
+            fused_caseb(&a, F.qb, &w, b, GROUP, &bacc);
+        }
+    }
+}
+
+template <bool COMMIT>
+__global__ void __launch_bounds__(kBatchedThreads, 3) fused_cell_kernel(const __grid_constant__ StepArgs a,
+                                                                        const __grid_constant__ FusedArgs F)
+{
+    __shared__ FusedWarp work[kFusedWarps];
+    __shared__ int staged[kFusedWarps];
+    __shared__ BlockAcc bacc;
+    block_acc_init(bacc);
+    __syncthreads();
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    FusedWarp& w = work[wid];
+    const int nwarps = gridDim.x * kFusedWarps;
+    int cell = blockIdx.x * kFusedWarps + wid;
+    for (int lead = blockIdx.x * kFusedWarps; lead < a.n_cells; lead += kFusedBatch * nwarps) {   // lead: warp 0's cell
+        const int first = cell;
+        int nq = 0, nb = 0;
+        if (lane < 3 * kFusedBatch) (&w.ev[0][0])[lane] = make_float2(0.f, 0.f);
+        if (lane == 0) w.changed = 0u;
+        __syncwarp();
+        for (; cell < a.n_cells && nb < kFusedBatch; cell += nwarps, ++nb) {
+            const int nt = a.ion.count[cell], t0 = a.ion.start[cell], mat = a.mat_of_cell[cell];
+            const int ne = F.run & 1u ? a.em.count[cell] : 0, np = F.run & 2u ? a.ep.count[cell] : 0,
+                      ng = F.run & 4u ? a.ph.count[cell] : 0;
+            const int e0 = a.em.start[cell], b0 = a.ep.start[cell], g0 = a.ph.start[cell];
+            if (lane == 0) {
+                w.cell[nb].cell = cell; w.cell[nb].t0 = t0; w.cell[nb].mat = mat; w.cell[nb].Nt = (uint32_t)nt;
+            }
+            if (nt <= 0 || (ne <= 0 && np <= 0 && ng <= 0)) continue;
+            if ((unsigned)mat >= (unsigned)a.n_mat) {
+                if (lane == 0) atomicOr(&bacc.status, PCC_ST_NONFINITE);
+                continue;
+            }
+            IonSums is;
+            is.have = false;
+            if (ne > 0) fused_scan<kGroupEm>(a, F, w, nb, cell, e0, ne, t0, nt, mat, is, nq, lane, bacc);
+            if (np > 0) fused_scan<kGroupEp>(a, F, w, nb, cell, b0, np, t0, nt, mat, is, nq, lane, bacc);
+            if (ng > 0) fused_scan<kGroupPh>(a, F, w, nb, cell, g0, ng, t0, nt, mat, is, nq, lane, bacc);
+        }
+        if (lane == 0) staged[wid] = nq;
+        __syncthreads();
+        fused_drain_block(&a, work, staged, &bacc);
+        __syncthreads();
+        for (unsigned ch = w.changed; ch; ch &= ch - 1u) {
+            const int b = (__ffs(ch) - 1) >> 2;
+            fused_finish(&a, &w, b);
+            ch &= ~(0xFu << (4 * b)) | (ch & -ch);   // the cell's other groups are done with it
+        }
+        if (COMMIT) {   // a lane per species of each cell; most have nothing to commit
+            __syncwarp();
+            if (lane < 3 * nb) {
+                const int b = lane / 3, sp = lane - 3 * b, c = first + b * nwarps;
+                if ((sp == 0 ? a.em.added : sp == 1 ? a.ep.added : a.ph.added)[c]) fused_commit(&a, sp, c);
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    block_acc_flush(bacc, a.st);
 }
 
 // Pairing diagnostic: one warp per cell.
@@ -2223,8 +2632,33 @@ static void warm_occupancy(pcc_ctx* ctx, int stage)
     persistent_grid(ctx, (const void*)caseb_cand_kernel<GROUP>, stage, 0);
 }
 
+// The fused kernel takes the call's cells whole: chosen where launches bound
+// the step (see kFusedCellsPerWarp).  A call with timing events between the groups
+// needs them apart, a context with its own wait limit asks for the staged
+// copies that the limit is about, and calls of a few cells keep the general
+// sequence, whose launch count callers can rely on.
+static bool use_fused(const pcc_ctx* ctx, int n_cells, int precision, bool split)
+{
+    return precision == PCC_FP32_BATCHED && !split && n_cells >= kFusedMinCells &&
+           n_cells <= kFusedCellsPerWarp * kFusedWarpsPerSM * ctx->num_sms && ctx->wait_polls == kWaitPolls;
+}
+
+template <bool COMMIT>
+static void launch_fused(pcc_ctx* ctx, const StepArgs& a, unsigned run, cudaStream_t st)
+{
+    FusedArgs F;
+    for (int g = 0; g < 3; ++g)
+        for (int i = 0; i < 4; ++i) F.thr[g][i] = ctx->scan_thr[g][i];
+    F.run = run;
+    F.qb = (uint32_t*)ctx->queue_b;
+    const int g = std::min(persistent_grid(ctx, (const void*)fused_cell_kernel<COMMIT>, 0, 0),
+                           (a.n_cells + kFusedWarps - 1) / kFusedWarps);
+    fused_cell_kernel<COMMIT><<<g, kBatchedThreads, 0, st>>>(a, F);
+    note_launches(1);
+}
+
 int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em, const pcc_species* ep,
-                    const pcc_species* ph, const pcc_species* ion, unsigned mask, int precision)
+                    const pcc_species* ph, const pcc_species* ion, unsigned mask, int precision, bool split)
 {
     if (!ctx || !cells || !em || !ep || !ph || !ion || cells->n_cells < 1) {
         set_error("pcc_collide: invalid argument");
@@ -2241,6 +2675,11 @@ int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em,
     const bool ei = (mask & (PCC_BREMS | PCC_TRIDENT)) != 0, bh = (mask & PCC_BH) != 0;
     const bool run_em = ei && (groups & PCC_GROUP_EM), run_ep = ei && (groups & PCC_GROUP_EP);
     const bool run_ph = bh && (groups & PCC_GROUP_PH);
+    if (use_fused(ctx, cells->n_cells, precision, split)) {
+        persistent_grid(ctx, (const void*)fused_cell_kernel<false>, 0, 0);
+        persistent_grid(ctx, (const void*)fused_cell_kernel<true>, 0, 0);
+        return ensure_queue(ctx, 0, std::max<size_t>((size_t)ion->capacity, 1));
+    }
     int rc = ensure_lists(ctx, cells->n_cells);
     if (rc) return rc;
     size_t cap_a = 0;
@@ -2305,7 +2744,8 @@ extern "C" int pcc_set_schedule(pcc_ctx* ctx, int min_blocks_per_sm, int blocks_
 
 int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_species* ep, pcc_species* ph,
                    const pcc_species* ion, double dt, uint64_t seed, uint64_t step, unsigned mask, int precision,
-                   float* ledger, cudaStream_t st, int (*after_group)(void* user, int group), void* user)
+                   float* ledger, cudaStream_t st, int (*after_group)(void* user, int group), void* user,
+                   bool* committed)
 {
     if (!ctx || !cells || !cells->material_of_cell || cells->n_cells < 1) {
         set_error("pcc_collide: invalid cells");
@@ -2333,8 +2773,19 @@ int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_sp
     const bool run[3] = {run_em, run_ep, run_ph};
     int stage = 0;
     if (precision == PCC_FP32_BATCHED) {
-        int rc = collide_prepare(ctx, cells, em, ep, ph, ion, mask, precision);
+        const bool split = after_group != nullptr;
+        int rc = collide_prepare(ctx, cells, em, ep, ph, ion, mask, precision, split);
         if (rc) return rc;
+        if (use_fused(ctx, cells->n_cells, precision, split)) {
+            cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return cuda_fail(e, "pcc_collide: launch");
+            const unsigned run_bits = (run_em ? 1u : 0u) | (run_ep ? 2u : 0u) | (run_ph ? 4u : 0u);
+            if (committed) launch_fused<true>(ctx, a, run_bits, st);
+            else if (run_bits) launch_fused<false>(ctx, a, run_bits, st);
+            if (committed) *committed = true;
+            e = cudaGetLastError();
+            return e == cudaSuccess ? PCC_OK : cuda_fail(e, "pcc_collide: launch");
+        }
         launch_class_sort(ctx, a, (run_em ? 1u : 0u) | (run_ep ? 2u : 0u) | (run_ph ? 4u : 0u), st);
         stage = table_stage_bytes(ctx);
     }
@@ -2368,7 +2819,7 @@ extern "C" int pcc_collide(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em
                            int precision, float* ledger, void* stream)
 {
     return collide_groups(ctx, cells, em, ep, ph, ion, dt, seed, step, mask, precision, ledger, (cudaStream_t)stream,
-                          nullptr, nullptr);
+                          nullptr, nullptr, nullptr);
 }
 
 extern "C" int pcc_pairing(pcc_ctx* ctx, int n_cells, const pcc_species* proj, const pcc_species* targ, int group,

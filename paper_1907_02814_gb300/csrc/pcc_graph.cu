@@ -45,14 +45,18 @@ static int after_group(void* user, int g)
 
 // One step on the capture stream: the groups of the mask one by one (the
 // batched path's class sort of all groups comes first, inside the first
-// part), then the three commits, with an event before and after each part.
+// part), then the three commits, with an event before and after each part
+// when timing was asked for; without events the call may run, commits
+// included, as one kernel.
 static int capture_step(pcc_ctx* ctx, const pcc_step_desc* d, uint64_t step, int s, cudaStream_t cs)
 {
     GroupEvents ev{ctx, 5 * s, cs};
+    bool committed = false;
     int rc = record(ctx, 5 * s, cs);
     if (rc == PCC_OK)
         rc = collide_groups(ctx, d->cells, d->em, d->ep, d->ph, d->ion, d->dt, d->seed, step, d->mask, d->precision,
-                            d->ledger, cs, after_group, &ev);
+                            d->ledger, cs, ctx->graph_events.empty() ? nullptr : after_group, &ev, &committed);
+    if (committed) return rc;
     if (rc == PCC_OK) rc = pcc_append_secondaries(ctx, d->cells->n_cells, d->em, cs);
     if (rc == PCC_OK) rc = pcc_append_secondaries(ctx, d->cells->n_cells, d->ep, cs);
     if (rc == PCC_OK) rc = pcc_append_secondaries(ctx, d->cells->n_cells, d->ph, cs);
@@ -69,7 +73,7 @@ extern "C" int pcc_steps_capture(pcc_ctx* ctx, const pcc_step_desc* d, uint64_t 
     }
     pcc_free_graph(ctx);
     // every allocation and occupancy query of the step happens here, outside the capture
-    int rc = collide_prepare(ctx, d->cells, d->em, d->ep, d->ph, d->ion, d->mask, d->precision);
+    int rc = collide_prepare(ctx, d->cells, d->em, d->ep, d->ph, d->ion, d->mask, d->precision, timing != 0);
     if (rc) return rc;
     cudaError_t e = cudaSuccess;
     if (!ctx->capture_stream) e = cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking);

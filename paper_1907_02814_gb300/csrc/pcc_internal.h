@@ -9,6 +9,8 @@
 #include "../../include/pcc.h"
 #include "pcc_device.cuh"
 
+namespace pcc { constexpr int kWaitPolls = 1 << 22; }
+
 struct pcc_ctx {
     int device = 0;
     int num_sms = 0;
@@ -51,7 +53,7 @@ struct pcc_ctx {
     int scan_thr[3][4] = {{20, 20, 15, 2}, {12, 12, 6, 0}, {17, 17, 15, 13}};
     int blocks_per_sm = 0;         // persistent grid cap (0: as many as fit)
     bool class_smem_ready = false; // large shared memory enabled for the class-sort offsets
-    int wait_polls = 1 << 22;      // bounded waits give up after this many polls (fault injection: 0)
+    int wait_polls = pcc::kWaitPolls;   // bounded waits give up after this many polls (fault injection: 0)
     // resident blocks per SM of the persistent kernels, by (kernel, dynamic smem)
     struct Occ { const void* fn; int smem; int per_sm; };
     std::vector<Occ> occ;
@@ -87,16 +89,19 @@ TableGeom make_geom(const pcc_table_spec& s);
 
 // Buffers and launch geometry of a pcc_collide call with these arguments,
 // set up ahead (allocations, occupancy queries) so the call itself can be
-// captured into a graph.
+// captured into a graph.  split: the groups are wanted one by one.
 int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em, const pcc_species* ep,
-                    const pcc_species* ph, const pcc_species* ion, unsigned mask, int precision);
+                    const pcc_species* ph, const pcc_species* ion, unsigned mask, int precision, bool split);
 // The work of pcc_collide on stream st.  After the kernels of group g
 // (0 e-, 1 e+, 2 photons) are enqueued, whether or not the group runs,
 // after_group(user, g) is called if given, so that a caller can record
 // events between the groups; a non-zero return ends the call with it.  The
 // batched path sorts the cells of every group that runs by size class
-// before the first group.
+// before the first group; without after_group it may run every group in one
+// kernel.  committed, if given, lets that kernel commit the secondaries too
+// and is set when it did.
 int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_species* ep, pcc_species* ph,
                    const pcc_species* ion, double dt, uint64_t seed, uint64_t step, unsigned mask, int precision,
-                   float* ledger, cudaStream_t st, int (*after_group)(void* user, int group), void* user);
+                   float* ledger, cudaStream_t st, int (*after_group)(void* user, int group), void* user,
+                   bool* committed);
 void pcc_free_graph(pcc_ctx* ctx);
