@@ -189,8 +189,8 @@ int pcc_tables_read(pcc_ctx *ctx, double *brems_sigma, double *brems_cdf, double
  * into the cell-region layout of `out`, each cell's particles in ascending
  * pid order.  Region of cell c: count_c + max(slack_abs, ceil(slack_rel *
  * count_c)) slots.  out->cell_start/cell_count/cell_added are written;
- * cell_added is zeroed.  Synchronises the stream (it reads back the
- * largest cell); PCC_E_CAPACITY if the regions do not fit out->capacity or
+ * cell_added is zeroed.  Waits until the counts are known (it reads back the
+ * largest cell), not for the records to arrive; PCC_E_CAPACITY if the regions do not fit out->capacity or
  * a cell holds more than 16384 particles. */
 int pcc_bin(pcc_ctx *ctx, const pcc_particles *in, int n_cells, pcc_species *out,
             int slack_abs, double slack_rel, void *stream);

@@ -100,6 +100,8 @@ extern "C" void pcc_destroy(pcc_ctx* ctx)
     pcc_free_tables(ctx);
     if (ctx->stats) cudaFree(ctx->stats);
     if (ctx->scratch) cudaFree(ctx->scratch);
+    if (ctx->bin_host) cudaFreeHost(ctx->bin_host);
+    if (ctx->bin_event) cudaEventDestroy(ctx->bin_event);
     if (ctx->lists) cudaFree(ctx->lists);
     if (ctx->queue_a) cudaFree(ctx->queue_a);
     if (ctx->queue_b) cudaFree(ctx->queue_b);

@@ -37,6 +37,9 @@ struct pcc_ctx {
     // scratch
     void* scratch = nullptr;
     size_t scratch_bytes = 0;
+    // pcc_bin: pinned copy of the totals and the event of its arrival
+    void* bin_host = nullptr;
+    cudaEvent_t bin_event = nullptr;
     // cell work lists of the batched collision kernels (3 groups + class counters)
     int* lists = nullptr;
     int lists_cells = 0;
