@@ -470,126 +470,268 @@ __device__ __forceinline__ void ei_pair(const StepArgs* ap, const Tab<Real>& tb,
     }
 }
 
-// Cell sums of Sec. III.A: n_p = sum W_p, n_t = sum W_t and
-// n_pt = sum over pairs of min(W_p, W_t).  One pass over both lists; when
-// every target of the cell has the same weight, a projectile's pairs all
-// contribute min(W_p, W_t), so n_pt needs no permutation.
-template <typename Real, class G>
-__device__ __forceinline__ void cell_sums(const G& grp, const SpeciesView& P, const SpeciesView& I, int p0, int t0,
-                                          uint32_t Np, uint32_t Nt, const Pairing& pr, Real& n_p, Real& n_t,
-                                          Real& n_pt)
+// ---- plain FP64: one block per cell ----------------------------------------------
+// Every decision is the FP64 one.  A pair is evaluated in full (frame, cross
+// section, acceptance: some 300 FP64 instructions, of which this chip issues
+// about two per clock and SM) only where that can matter: its accept digit
+// passes a bound on the acceptance probability (exact, as in the batched path:
+// x <= coef B, and p <= x), or its energy, by a float bound with a margin, may lie
+// above the tables, or its momentum is not plainly finite, so that the status
+// bits come out as if every pair were evaluated.  A step of 16384 Au cells of 256
+// electrons, 64 ions and 64 photons takes 0.55 ms (3.59 ms with every pair
+// evaluated), bound by the latency of a block's phases.
+constexpr int kPlainThreads = 128, kPlainWarps = kPlainThreads / 32;
+
+// Per-block counters, updated with shared atomics and added to the context's
+// counters once per block.
+struct BlockAcc {
+    unsigned long long pairs[3], accepted[5], created[5], candidates[3];
+    double dE;
+    unsigned status;
+};
+
+__device__ __forceinline__ void block_acc_init(BlockAcc& b)
 {
-    const float w0 = I.w[t0];
-    Real sp = 0, st = 0, sf = 0;
-    float wmin = w0, wmax = w0;
-    const uint32_t N = Np > Nt ? Np : Nt;
-#pragma unroll 4
-    for (uint32_t s = grp.rank(); s < N; s += grp.size()) {
-        if (s < Nt) {
-            const float wt = I.w[t0 + s];
-            st += (Real)wt;
-            wmin = fminf(wmin, wt);
-            wmax = fmaxf(wmax, wt);
-        }
-        if (s < Np) {
-            const float wp = P.w[p0 + s];
-            sp += (Real)wp;
-            const uint32_t npairs = pr.caseA ? 1u : (Nt - s + Np - 1) / Np;
-            sf += (Real)fminf(wp, w0) * (Real)npairs;
-        }
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 3; ++i) b.pairs[i] = b.candidates[i] = 0;
+        for (int i = 0; i < 5; ++i) b.accepted[i] = b.created[i] = 0;
+        b.dE = 0.0;
+        b.status = 0;
     }
-    n_p = grp.sum(sp);
-    n_t = grp.sum(st);
-    const float lo = grp.fmin(wmin), hi = grp.fmax(wmax);
-    if (lo == hi) {
-        n_pt = grp.sum(sf);
-        return;
-    }
-    Real spt = 0;
-    for (uint32_t s = grp.rank(); s < Np; s += grp.size()) {
-        const float wp = P.w[p0 + s];
-        if (pr.caseA) {
-            spt += (Real)fminf(wp, I.w[t0 + pr.pair_of_slot(s) % Nt]);
-        } else {
-            for (uint32_t j = s; j < Nt; j += Np) spt += (Real)fminf(wp, I.w[t0 + pr.target_of_pair(j)]);
-        }
-    }
-    n_pt = grp.sum(spt);
 }
 
-// ---- one cell of electron (or positron) - ion pairs ---------------------------
-template <typename Real, class G>
-__device__ void ei_cell(const G& grp, const StepArgs* ap, const Tab<Real>& tb, int group, int cell, Acc& acc)
+__device__ __forceinline__ void block_acc_flush(const BlockAcc& b, DevStats* st)
+{
+    if (threadIdx.x != 0) return;
+    for (int i = 0; i < 3; ++i) {
+        if (b.pairs[i]) atomicAdd(&st->pairs[i], b.pairs[i]);
+        if (b.candidates[i]) atomicAdd(&st->candidates[i], b.candidates[i]);
+    }
+    for (int i = 0; i < 5; ++i) {
+        if (b.accepted[i]) atomicAdd(&st->accepted[i], b.accepted[i]);
+        if (b.created[i]) atomicAdd(&st->created[i], b.created[i]);
+    }
+    if (b.dE != 0.0) atomicAdd(&st->energy_change, b.dE);
+    if (b.status) atomicOr(&st->status, b.status);
+}
+
+// A thread's counters to the block's.
+__device__ __forceinline__ void add_rare(const Acc& acc, BlockAcc& b)
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        if (acc.accepted[i]) atomicAdd(&b.accepted[i], (unsigned long long)acc.accepted[i]);
+        if (acc.created[i]) atomicAdd(&b.created[i], (unsigned long long)acc.created[i]);
+    }
+    if (acc.dE != 0.0) atomicAdd(&b.dE, acc.dE);
+    if (acc.status) atomicOr(&b.status, acc.status);
+}
+
+struct PlainShared {
+    BlockAcc acc;
+    int scratch[64];                  // pairing tables of short lists
+    double sum[3][kPlainWarps];
+    float lo[kPlainWarps], hi[kPlainWarps], fac[kPlainWarps];
+    double red[kPlainWarps];
+};
+
+// What a block knows of its cell.
+struct PlainCell {
+    int cell, mat, p0, t0;
+    uint32_t Np, Nt;
+    Pairing pr;
+    double coef, fac;                 // fac: 1 + max |beta_i| rounded up, for the digit bounds
+    float reach2;                     // (gamma_i + |u_i|)^2 at its largest, rounded up: gamma' <= gamma sqrt(reach2)
+};
+
+// Cell sums of Sec. III.A (n_p = sum W_p, n_t = sum W_t, n_pt = sum over pairs of
+// min(W_p, W_t)) and the largest ion speed.  One pass over both lists; when every
+// target of the cell has the same weight, a projectile's pairs all contribute
+// min(W_p, W_t), so n_pt needs no permutation.  Threads over the lists in
+// strides of the block, then warps by butterflies, then the warps in order.
+__device__ __forceinline__ void plain_sums(const CtaGroup& grp, PlainShared& S, const StepArgs& a, const SpeciesView& P,
+                                           PlainCell& c)
+{
+    const SpeciesView& I = a.ion;
+    const uint32_t Np = c.Np, Nt = c.Nt;
+    const float w0 = I.w[c.t0];
+    double sp = 0, st = 0, sf = 0;
+    float wmin = w0, wmax = w0, u2m = 0.f, u2s = 0.f;
+    for (uint32_t s = threadIdx.x; s < Nt; s += kPlainThreads) {
+        const int t = c.t0 + (int)s;
+        const float wt = I.w[t], ux = I.ux[t], uy = I.uy[t], uz = I.uz[t];
+        st += (double)wt;
+        wmin = fminf(wmin, wt);
+        wmax = fmaxf(wmax, wt);
+        const float u2 = ux * ux + uy * uy + uz * uz;
+        u2m = fmaxf(u2m, u2);
+        u2s += u2;
+    }
+    if (c.pr.caseA) {
+#pragma unroll 4
+        for (uint32_t s = threadIdx.x; s < Np; s += kPlainThreads) {
+            const float wp = P.w[c.p0 + (int)s];
+            sp += (double)wp;
+            sf += (double)fminf(wp, w0);
+        }
+    } else {
+        for (uint32_t s = threadIdx.x; s < Np; s += kPlainThreads) {
+            const float wp = P.w[c.p0 + (int)s];
+            sp += (double)wp;
+            sf += (double)fminf(wp, w0) * (double)((Nt - s + Np - 1) / Np);
+        }
+    }
+    // gamma_i + |u_i| and beta_i grow with u_i^2; a u^2 past 1e12, or a momentum
+    // that is not finite, makes the reach infinite (every pair is evaluated)
+    sp = warp_sum(sp);
+    st = warp_sum(st);
+    sf = warp_sum(sf);
+    if (!(u2s < 1e12f)) u2m = __int_as_float(0x7f800000);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        wmin = fminf(wmin, __shfl_xor_sync(0xffffffffu, wmin, o));
+        wmax = fmaxf(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+        u2m = fmaxf(u2m, __shfl_xor_sync(0xffffffffu, u2m, o));
+    }
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) {
+        S.sum[0][w] = sp; S.sum[1][w] = st; S.sum[2][w] = sf;
+        S.lo[w] = wmin; S.hi[w] = wmax; S.fac[w] = u2m;
+    }
+    __syncthreads();
+    double n_p = 0, n_t = 0, n_pt = 0;
+    float lo = S.lo[0], hi = S.hi[0], um = 0.f;
+    for (int k = 0; k < kPlainWarps; ++k) {
+        n_p += S.sum[0][k];
+        n_t += S.sum[1][k];
+        n_pt += S.sum[2][k];
+        lo = fminf(lo, S.lo[k]);
+        hi = fmaxf(hi, S.hi[k]);
+        um = fmaxf(um, S.fac[k]);
+    }
+    const float ui = sqrtf(um), gi = sqrtf(1.f + um);
+    c.reach2 = (gi + ui) * (gi + ui) * 1.0001f;
+    c.fac = um < 1e12f ? 1.0 + (double)fminf(ui / gi * 1.0001f, 1.f) : 2.0;
+    if (!(lo == hi)) {
+        double spt = 0;
+        for (uint32_t s = threadIdx.x; s < Np; s += kPlainThreads) {
+            const float wp = P.w[c.p0 + (int)s];
+            if (c.pr.caseA) {
+                spt += (double)fminf(wp, I.w[c.t0 + c.pr.pair_of_slot(s) % Nt]);
+            } else {
+                for (uint32_t j = s; j < Nt; j += Np) spt += (double)fminf(wp, I.w[c.t0 + c.pr.target_of_pair(j)]);
+            }
+        }
+        n_pt = grp.sum(spt);
+    }
+    c.coef = (n_p / n_pt) * n_t * (double)(kC * a.dt);
+}
+
+// Digit threshold of the bound x <= coef bound_2 fac / 2, where bound_2 (for
+// 1 + |beta_i| = 2) carries a margin of 1e-3.
+__device__ __forceinline__ uint32_t plain_threshold(const PlainCell& c, float bound)
+{
+    const double X = c.coef * (double)bound * (0.5 * c.fac) * 65536.0;
+    if (!(X < 65535.0)) return 0xFFFFu;
+    return X > 0.0 ? (uint32_t)X : 0u;
+}
+
+// Sets up the block's cell; false when it has no pairs (uniform over the block).
+__device__ __forceinline__ bool plain_cell(const CtaGroup& grp, PlainShared& S, const StepArgs& a, const SpeciesView& P,
+                                           int group, int cell, PlainCell& c)
+{
+    c.cell = cell;
+    c.Np = P.count[cell];
+    c.Nt = a.ion.count[cell];
+    if (c.Np == 0 || c.Nt == 0) return false;
+    block_acc_init(S.acc);
+    __syncthreads();
+    c.p0 = P.start[cell];
+    c.t0 = a.ion.start[cell];
+    c.mat = a.mat_of_cell[cell];
+    if ((unsigned)c.mat >= (unsigned)a.n_mat) {
+        if (threadIdx.x == 0) S.acc.status |= PCC_ST_NONFINITE;
+        block_acc_flush(S.acc, a.st);
+        return false;
+    }
+    c.pr = make_pairing(grp, c.Np, c.Nt, cell, group, a);
+    plain_sums(grp, S, a, P, c);
+    const uint32_t Npair = c.Np > c.Nt ? c.Np : c.Nt;
+    if (threadIdx.x == 0) {
+        S.acc.pairs[group] += Npair;
+        if (Npair > 65536u || (uint32_t)cell > 0xFFFFFFu || a.step > 0x7FFFFull) atomicOr(&S.acc.status, PCC_ST_ID_RANGE);
+    }
+    return true;
+}
+
+// Whether energies up to sqrt(e2 reach2) stay below `limit` (e2: gamma^2 or k^2 in
+// FP32, not NaN) with a margin for the float arithmetic.
+__device__ __forceinline__ bool plainly_below(float e2, float reach2, float limit)
+{
+    return e2 < 1e30f && e2 * reach2 < limit * limit * 0.9999f;
+}
+
+// Evaluates one electron (positron) - ion pair in full.  Out of line: it takes
+// most of a block's registers and few pairs need it.  ev: radiated energy and
+// created weight.  True when the projectile changed.
+__device__ __noinline__ bool plain_ei_pair(const StepArgs* ap, int group, const PlainCell* cp, uint32_t s, uint32_t j,
+                                           uint32_t t, uint32_t rB, uint32_t rT, uint32_t pass, BlockAcc* bacc, float2* ev)
 {
     const StepArgs& a = *ap;
     const SpeciesView& P = group == kGroupEm ? a.em : a.ep;
-    const SpeciesView& I = a.ion;
-    const uint32_t Np = P.count[cell], Nt = I.count[cell];
-    if (Np == 0 || Nt == 0) return;
-    const int p0 = P.start[cell], t0 = I.start[cell];
-    const int mat = a.mat_of_cell[cell];
-    if ((unsigned)mat >= (unsigned)a.n_mat) {
-        acc.status |= PCC_ST_NONFINITE;
-        return;
+    const Tab<double> tb{a.brems_sigma, a.brems_cdf, a.bh_sigma, a.bh_cdf, a.tri_gp, a.tri_split};
+    const int sl = cp->p0 + (int)s;
+    float u[3] = {P.ux[sl], P.uy[sl], P.uz[sl]};
+    const float w = P.w[sl], xp = P.x ? P.x[sl] : 0.f;
+    const double Zf = a.screen[(size_t)cp->mat * kScreenFields + 7];
+    const AcceptSrc src{2 * s, (uint32_t)cp->cell, stream_tag(group, kAcceptExt, pass)};
+    Acc acc;
+    acc.zero();
+    bool dirty = false;
+    ei_pair<double>(ap, tb, group, cp->cell, cp->mat, Zf, cp->coef, u, &w, xp, cp->t0 + (int)t, j, rB, rT, src, acc, ev->x,
+                    ev->y, dirty);
+    if (dirty) {
+        P.ux[sl] = u[0]; P.uy[sl] = u[1]; P.uz[sl] = u[2];
     }
-    const Pairing pr = make_pairing(grp, Np, Nt, cell, group, a);
-    Real n_p, n_t, n_pt;
-    cell_sums<Real>(grp, P, I, p0, t0, Np, Nt, pr, n_p, n_t, n_pt);
-    const Real coef = (n_p / n_pt) * n_t * (Real)(kC * a.dt);
-    const uint32_t Npair = Np > Nt ? Np : Nt;
-    if (grp.rank() == 0) acc.pairs[group] += Npair;
-    if (Npair > 65536u || (uint32_t)cell > 0xFFFFFFu || a.step > 0x7FFFFull) acc.status |= PCC_ST_ID_RANGE;
-    const Real Zf = sizeof(Real) == 8 ? (Real)a.screen[(size_t)mat * kScreenFields + 7] : (Real)a.f_Z[mat];
-    // the FP32 path rejects from the accept digits alone above the bounds
-    const bool quick = sizeof(Real) == 4;
-    const uint32_t kB = quick && (a.mask & PCC_BREMS) ? accept_threshold((float)(coef * (Real)a.f_bound[3 * mat])) : 0u;
-    const uint32_t kT =
-        quick && (a.mask & PCC_TRIDENT) ? accept_threshold((float)(coef * (Real)a.f_bound[3 * mat + 1])) : 0u;
-    float rad = 0.f, wcre = 0.f;
+    add_rare(acc, *bacc);
+    return dirty;
+}
+
+__device__ void plain_ei_cell(const CtaGroup& grp, PlainShared& S, const StepArgs& a, int group, int cell)
+{
+    const SpeciesView& P = group == kGroupEm ? a.em : a.ep;
+    PlainCell c;
+    if (!plain_cell(grp, S, a, P, group, cell, c)) return;
+    const uint32_t kB = a.mask & PCC_BREMS ? plain_threshold(c, a.f_bound[3 * c.mat]) : 0u;
+    const uint32_t kT = a.mask & PCC_TRIDENT ? plain_threshold(c, a.f_bound[3 * c.mat + 1]) : 0u;
+    // the Trident bound holds to gamma' = 1e7
+    const float limit = (float)fmin(a.g.T_max + 1.0, 1e7);
+    float2 ev = make_float2(0.f, 0.f);
     bool had = false;
-    const bool has_x = P.x != nullptr;
     // two 16-bit accept digits per pair (Brems, Trident): slots 4q .. 4q + 3
     // share the draw of counter q, slot 4q + h its digits 2h and 2h + 1.  A
     // thread per slot (each takes its own copy of the draw), so that small
     // cells keep their threads busy.
-    for (uint32_t s = grp.rank(); s < Np; s += grp.size()) {
+    for (uint32_t s = threadIdx.x; s < c.Np; s += kPlainThreads) {
         const uint32_t q = s >> 2, h = s & 3u;
-        {
-            const int sl = p0 + (int)s;
-            float u[3] = {P.ux[sl], P.uy[sl], P.uz[sl]};
-            const float w = P.w[sl];
-            const float xp = has_x ? P.x[sl] : 0.f;
-            bool dirty = false;
-            if (pr.caseA) {
-                const uint32_t j = pr.pair_of_slot(s);
-                const Philox4 ac = draw(q, cell, a.step, stream_tag(group, kAccept, 0), a.seed);
-                const uint32_t rB = accept_digit(ac, 2 * h), rT = accept_digit(ac, 2 * h + 1);
-                if (!quick || rB <= kB || rT <= kT) {
-                    if (quick) acc.candidates[group]++;
-                    const AcceptSrc src{8 * q + 2 * h, (uint32_t)cell, stream_tag(group, kAcceptExt, 0)};
-                    ei_pair<Real>(ap, tb, group, cell, mat, Zf, coef, u, &w, xp, t0 + (int)(j % Nt), j, rB, rT, src,
-                                  acc, rad, wcre, dirty);
-                }
-            } else {
-                for (uint32_t m = 0, j = s; j < Nt; ++m, j += Np) {
-                    const Philox4 am = draw(q, cell, a.step, stream_tag(group, kAccept, m), a.seed);
-                    const uint32_t rB = accept_digit(am, 2 * h), rT = accept_digit(am, 2 * h + 1);
-                    if (quick && !(rB <= kB || rT <= kT)) continue;
-                    acc.candidates[group]++;
-                    const AcceptSrc src{8 * q + 2 * h, (uint32_t)cell, stream_tag(group, kAcceptExt, m)};
-                    ei_pair<Real>(ap, tb, group, cell, mat, Zf, coef, u, &w, xp, t0 + (int)pr.target_of_pair(j), j,
-                                  rB, rT, src, acc, rad, wcre, dirty);
-                }
-            }
-            if (dirty) {
-                P.ux[sl] = u[0]; P.uy[sl] = u[1]; P.uz[sl] = u[2];
-                had = true;
-            }
+        const int sl = c.p0 + (int)s;
+        const float ux = P.ux[sl], uy = P.uy[sl], uz = P.uz[sl];
+        const bool below = plainly_below(1.f + (ux * ux + uy * uy + uz * uz), c.reach2, limit);
+        const uint32_t passes = c.pr.caseA ? 1u : (c.Nt - s + c.Np - 1) / c.Np;
+        for (uint32_t m = 0; m < passes; ++m) {
+            const Philox4 ac = draw_k(q, cell, (uint32_t)a.step, stream_tag(group, kAccept, m), a.keys);
+            const uint32_t rB = accept_digit(ac, 2 * h), rT = accept_digit(ac, 2 * h + 1);
+            if (below && rB > kB && rT > kT) continue;
+            const uint32_t j = c.pr.caseA ? c.pr.pair_of_slot(s) : s + m * c.Np;
+            const uint32_t t = c.pr.caseA ? j % c.Nt : c.pr.target_of_pair(j);
+            had |= plain_ei_pair(&a, group, &c, s, j, t, rB, rT, m, &S.acc, &ev);
         }
+        // the full path counts every pair of such a cell as a candidate
+        if (!c.pr.caseA) atomicAdd(&S.acc.candidates[group], (unsigned long long)passes);
     }
     if (a.ledger && grp.any(had)) {
-        const float r = grp.sum(rad), wc = grp.sum(wcre);
-        if (grp.rank() == 0) {
+        const float r = grp.sum(ev.x), wc = grp.sum(ev.y);
+        if (threadIdx.x == 0) {
             float4* L = reinterpret_cast<float4*>(a.ledger) + cell;
             float4 v = *L;
             Kahan k1{v.x, v.y}, k2{v.z, v.w};
@@ -598,98 +740,91 @@ __device__ void ei_cell(const G& grp, const StepArgs* ap, const Tab<Real>& tb, i
             *L = make_float4(k1.s, k1.c, k2.s, k2.c);
         }
     }
+    __syncthreads();
+    block_acc_flush(S.acc, a.st);
 }
 
-// ---- one cell of photon - ion pairs (Bethe-Heitler) ---------------------------
-template <typename Real, class G>
-__device__ void bh_cell(const G& grp, const StepArgs* ap, const Tab<Real>& tb, int cell, Acc& acc)
+// Evaluates one photon - ion pair in full: 1 absorbed (weight set to 0), 0 not,
+// -1 the photon's momentum is not finite (flagged).
+__device__ __noinline__ int plain_bh_pair(const StepArgs* ap, const PlainCell* cp, uint32_t s, uint32_t j, uint32_t tau,
+                                          uint32_t rw, uint32_t pass, BlockAcc* bacc, float* wcre)
 {
     const StepArgs& a = *ap;
     const SpeciesView& P = a.ph;
     const SpeciesView& I = a.ion;
-    const uint32_t Np = P.count[cell], Nt = I.count[cell];
-    if (Np == 0 || Nt == 0) return;
-    const int p0 = P.start[cell], t0 = I.start[cell];
-    const int mat = a.mat_of_cell[cell];
-    if ((unsigned)mat >= (unsigned)a.n_mat) {
-        acc.status |= PCC_ST_NONFINITE;
-        return;
-    }
-    const Pairing pr = make_pairing(grp, Np, Nt, cell, kGroupPh, a);
-    Real n_p, n_t, n_pt;
-    cell_sums<Real>(grp, P, I, p0, t0, Np, Nt, pr, n_p, n_t, n_pt);
-    const Real coef = (n_p / n_pt) * n_t * (Real)(kC * a.dt);
-    const uint32_t Npair = Np > Nt ? Np : Nt;
-    if (grp.rank() == 0) acc.pairs[kGroupPh] += Npair;
-    if (Npair > 65536u || (uint32_t)cell > 0xFFFFFFu || a.step > 0x7FFFFull) acc.status |= PCC_ST_ID_RANGE;
-    float wcre = 0.f;
-    bool absorbed_any = false;
-    const bool has_x = P.x != nullptr;
-    const bool quick = sizeof(Real) == 4;
-    const uint32_t kBH = quick ? accept_threshold((float)(coef * (Real)a.f_bound[3 * mat + 2])) : 0u;
-    // one 16-bit accept digit per pair (BH): slots 8q .. 8q + 7 share the
-    // draw of counter q, slot 8q + h its digit h; a thread per slot
-    for (uint32_t s = grp.rank(); s < Np; s += grp.size()) {
-        const uint32_t q = s >> 3, h = s & 7u;
-        {
-            const int sl = p0 + (int)s;
-            const uint32_t npass = pr.caseA ? 1u : (Nt - s + Np - 1) / Np;
-            bool loaded = false;
-            Real uk[3] = {0, 0, 0}, k = 0;
-            for (uint32_t m = 0; m < npass; ++m) {
-                uint32_t j, tau;
-                const uint32_t rw =
-                    accept_digit(draw(q, cell, a.step, stream_tag(kGroupPh, kAccept, m), a.seed), h);
-                if (quick && !(rw <= kBH)) continue;   // exact quick reject
-                if (pr.caseA) {
-                    j = pr.pair_of_slot(s);
-                    tau = j % Nt;
-                } else {
-                    j = s + m * Np;
-                    tau = pr.target_of_pair(j);
-                }
-                if (quick) acc.candidates[kGroupPh]++;
-                if (!loaded) {
-                    uk[0] = (Real)P.ux[sl]; uk[1] = (Real)P.uy[sl]; uk[2] = (Real)P.uz[sl];
-                    k = sqrt(uk[0] * uk[0] + uk[1] * uk[1] + uk[2] * uk[2]);
-                    loaded = true;
-                }
-                if (!isfinite(k)) { acc.status |= PCC_ST_NONFINITE; break; }
-                const int ts = t0 + (int)tau;
-                Frame<Real> f;
-                f.ui[0] = I.ux[ts]; f.ui[1] = I.uy[ts]; f.ui[2] = I.uz[ts];
-                f.gi = sqrt((Real)1 + f.ui[0] * f.ui[0] + f.ui[1] * f.ui[1] + f.ui[2] * f.ui[2]);
-                const Real d = f.ui[0] * uk[0] + f.ui[1] * uk[1] + f.ui[2] * uk[2];
-                const Real kp = f.gi * k - d;
-                const Real sig = sigma_at<Real>(tb, tb.hsig + (size_t)mat * a.g.n_rows, a.g, kp - (Real)2, acc.status);
-                if (!(sig > (Real)0)) continue;
-                const Real x = coef * sig * kp / (k * f.gi);
-                if (x > (Real)1) acc.status |= PCC_ST_PROB_LARGE;
-                const AcceptSrc src{8 * q + h, (uint32_t)cell, stream_tag(kGroupPh, kAcceptExt, m)};
-                if (!accept_u<Real>(rw, -expm1(-x), src, a.step, a.seed)) continue;
-                acc.accepted[kChBH]++;
-                const Real fac = d / (f.gi + (Real)1) - k;
-                const Real pv[3] = {uk[0] + fac * f.ui[0], uk[1] + fac * f.ui[1], uk[2] + fac * f.ui[2]};
-                const Real pm = sqrt(pv[0] * pv[0] + pv[1] * pv[1] + pv[2] * pv[2]);
-                f.n[0] = pv[0] / pm; f.n[1] = pv[1] / pm; f.n[2] = pv[2] / pm;
-                const float xpos = has_x ? P.x[sl] : 0.f;
-                const EventResult r = bh_event<Real>(ap, tb, cell, mat, j, P.w[sl], I.w[ts], xpos, f, kp, k);
-                if (!r.created) continue;
+    const Tab<double> tb{a.brems_sigma, a.brems_cdf, a.bh_sigma, a.bh_cdf, a.tri_gp, a.tri_split};
+    const int sl = cp->p0 + (int)s, ts = cp->t0 + (int)tau, cell = cp->cell, mat = cp->mat;
+    const double uk[3] = {P.ux[sl], P.uy[sl], P.uz[sl]};
+    const double k = sqrt(uk[0] * uk[0] + uk[1] * uk[1] + uk[2] * uk[2]);
+    if (!isfinite(k)) { atomicOr(&bacc->status, PCC_ST_NONFINITE); return -1; }
+    Frame<double> f;
+    f.ui[0] = I.ux[ts]; f.ui[1] = I.uy[ts]; f.ui[2] = I.uz[ts];
+    f.gi = sqrt(1.0 + f.ui[0] * f.ui[0] + f.ui[1] * f.ui[1] + f.ui[2] * f.ui[2]);
+    const double d = f.ui[0] * uk[0] + f.ui[1] * uk[1] + f.ui[2] * uk[2];
+    const double kp = f.gi * k - d;
+    Acc acc;
+    acc.zero();
+    const double sig = sigma_at<double>(tb, tb.hsig + (size_t)mat * a.g.n_rows, a.g, kp - 2.0, acc.status);
+    int absorbed = 0;
+    if (sig > 0.0) {
+        const double x = cp->coef * sig * kp / (k * f.gi);
+        if (x > 1.0) acc.status |= PCC_ST_PROB_LARGE;
+        const AcceptSrc src{s, (uint32_t)cell, stream_tag(kGroupPh, kAcceptExt, pass)};
+        if (accept_u<double>(rw, -expm1(-x), src, a.step, a.seed)) {
+            acc.accepted[kChBH]++;
+            const double fac = d / (f.gi + 1.0) - k;
+            const double pv[3] = {uk[0] + fac * f.ui[0], uk[1] + fac * f.ui[1], uk[2] + fac * f.ui[2]};
+            const double pm = sqrt(pv[0] * pv[0] + pv[1] * pv[1] + pv[2] * pv[2]);
+            f.n[0] = pv[0] / pm; f.n[1] = pv[1] / pm; f.n[2] = pv[2] / pm;
+            const float xpos = P.x ? P.x[sl] : 0.f;
+            const EventResult r = bh_event<double>(ap, tb, cell, mat, j, P.w[sl], I.w[ts], xpos, f, kp, k);
+            if (r.created) {
                 acc.created[kChBH]++;
                 acc.dE += r.dE;
                 acc.status |= r.status;
-                wcre += r.wc;
+                *wcre += r.wc;
                 P.w[sl] = 0.f;   // removal marker, compacted below; skips the photon's later pairs
-                absorbed_any = true;
-                break;
+                absorbed = 1;
             }
+        }
+    }
+    add_rare(acc, *bacc);
+    return absorbed;
+}
+
+__device__ void plain_bh_cell(const CtaGroup& grp, PlainShared& S, const StepArgs& a, int cell)
+{
+    const SpeciesView& P = a.ph;
+    PlainCell c;
+    if (!plain_cell(grp, S, a, P, kGroupPh, cell, c)) return;
+    const uint32_t kBH = plain_threshold(c, a.f_bound[3 * c.mat + 2]);
+    const float limit = (float)(a.g.T_max + 2.0);
+    float wcre = 0.f;
+    bool absorbed_any = false;
+    // one 16-bit accept digit per pair (BH): slots 8q .. 8q + 7 share the
+    // draw of counter q, slot 8q + h its digit h; a thread per slot
+    for (uint32_t s = threadIdx.x; s < c.Np; s += kPlainThreads) {
+        const uint32_t q = s >> 3, h = s & 7u;
+        const int sl = c.p0 + (int)s;
+        const float ux = P.ux[sl], uy = P.uy[sl], uz = P.uz[sl];
+        const bool below = plainly_below(ux * ux + uy * uy + uz * uz, c.reach2, limit);
+        const uint32_t passes = c.pr.caseA ? 1u : (c.Nt - s + c.Np - 1) / c.Np;
+        for (uint32_t m = 0; m < passes; ++m) {
+            const uint32_t rw =
+                accept_digit(draw_k(q, cell, (uint32_t)a.step, stream_tag(kGroupPh, kAccept, m), a.keys), h);
+            if (below && rw > kBH) continue;
+            const uint32_t j = c.pr.caseA ? c.pr.pair_of_slot(s) : s + m * c.Np;
+            const uint32_t tau = c.pr.caseA ? j % c.Nt : c.pr.target_of_pair(j);
+            const int r = plain_bh_pair(&a, &c, s, j, tau, rw, m, &S.acc, &wcre);
+            absorbed_any |= r > 0;
+            if (r) break;
         }
     }
     if (grp.any(absorbed_any)) {
         grp.sync();
         if (a.ledger) {
             const float wc = grp.sum(wcre);
-            if (grp.rank() == 0) {
+            if (threadIdx.x == 0) {
                 float4* L = reinterpret_cast<float4*>(a.ledger) + cell;
                 float4 v = *L;
                 Kahan k2{v.z, v.w};
@@ -697,12 +832,13 @@ __device__ void bh_cell(const G& grp, const StepArgs* ap, const Tab<Real>& tb, i
                 *L = make_float4(v.x, v.y, k2.s, k2.c);
             }
         }
-        if (grp.rank() == 0) {   // stable compaction of the region (rare path)
-            const int n_all = (int)Np + P.added[cell];
+        if (threadIdx.x == 0) {   // stable compaction of the region (rare path)
+            const bool has_x = P.x != nullptr;
+            const int Np = (int)c.Np, p0 = c.p0, n_all = Np + P.added[cell];
             int wr = 0, removed = 0;
             for (int i = 0; i < n_all; ++i) {
                 const int src = p0 + i;
-                if (i < (int)Np && P.w[src] == 0.f) { ++removed; continue; }
+                if (i < Np && P.w[src] == 0.f) { ++removed; continue; }
                 if (wr != i) {
                     const int dst = p0 + wr;
                     P.ux[dst] = P.ux[src]; P.uy[dst] = P.uy[src]; P.uz[dst] = P.uz[src]; P.w[dst] = P.w[src];
@@ -711,56 +847,20 @@ __device__ void bh_cell(const G& grp, const StepArgs* ap, const Tab<Real>& tb, i
                 }
                 ++wr;
             }
-            P.count[cell] = (int)Np - removed;
+            P.count[cell] = Np - removed;
         }
-        grp.sync();
     }
+    __syncthreads();
+    block_acc_flush(S.acc, a.st);
 }
 
-// ---- kernels --------------------------------------------------------------------
-__device__ void flush_acc(Acc& acc, DevStats* st, bool lane_reduce)
-{
-    unsigned long long pv[3];
-    unsigned av[5], cv[5], kv[3];
-    double dE = acc.dE, dQ = acc.dQ;
-    unsigned status = acc.status;
-    for (int i = 0; i < 3; ++i) pv[i] = acc.pairs[i], kv[i] = acc.candidates[i];
-    for (int i = 0; i < 5; ++i) { av[i] = acc.accepted[i]; cv[i] = acc.created[i]; }
-    if (lane_reduce) {
-        for (int i = 0; i < 3; ++i) pv[i] = warp_sum(pv[i]), kv[i] = warp_sum(kv[i]);
-        for (int i = 0; i < 5; ++i) { av[i] = warp_sum(av[i]); cv[i] = warp_sum(cv[i]); }
-        dE = warp_sum(dE);
-        dQ = warp_sum(dQ);
-        status = __reduce_or_sync(0xffffffffu, status);
-        if ((threadIdx.x & 31) != 0) return;
-    }
-    for (int i = 0; i < 3; ++i) {
-        if (pv[i]) atomicAdd(&st->pairs[i], pv[i]);
-        if (kv[i]) atomicAdd(&st->candidates[i], (unsigned long long)kv[i]);
-    }
-    for (int i = 0; i < 5; ++i) {
-        if (av[i]) atomicAdd(&st->accepted[i], (unsigned long long)av[i]);
-        if (cv[i]) atomicAdd(&st->created[i], (unsigned long long)cv[i]);
-    }
-    if (dE != 0.0) atomicAdd(&st->energy_change, dE);
-    if (dQ != 0.0) atomicAdd(&st->charge_change, dQ);
-    if (status) atomicOr(&st->status, status);
-}
-
-// Plain FP64: one block per cell.
 template <int GROUP>
-__global__ void __launch_bounds__(128) collide_plain_kernel(const __grid_constant__ StepArgs a)
+__global__ void __launch_bounds__(kPlainThreads, 8) collide_plain_kernel(const __grid_constant__ StepArgs a)
 {
-    __shared__ int scratch[64];
-    __shared__ double red[4];
-    CtaGroup grp{scratch, red};
-    Tab<double> tb{a.brems_sigma, a.brems_cdf, a.bh_sigma, a.bh_cdf, a.tri_gp, a.tri_split};
-    Acc acc;
-    acc.zero();
-    const int cell = blockIdx.x;
-    if (GROUP == kGroupPh) bh_cell<double>(grp, &a, tb, cell, acc);
-    else ei_cell<double>(grp, &a, tb, GROUP, cell, acc);
-    flush_acc(acc, a.st, true);
+    __shared__ PlainShared S;
+    const CtaGroup grp{S.scratch, S.red};
+    if (GROUP == kGroupPh) plain_bh_cell(grp, S, a, blockIdx.x);
+    else plain_ei_cell(grp, S, a, GROUP, blockIdx.x);
 }
 
 // Batched FP32 -----------------------------------------------------------------
@@ -1055,39 +1155,6 @@ __device__ __forceinline__ CellMeta load_meta(const StepArgs& a, const SpeciesVi
     m.t0 = a.ion.start[cell];
     m.mat = a.mat_of_cell[cell];
     return m;
-}
-
-// Per-block counters of the batched kernels, updated with shared atomics and
-// added to the context's counters once per block.
-struct BlockAcc {
-    unsigned long long pairs[3], accepted[5], created[5], candidates[3];
-    double dE;
-    unsigned status;
-};
-
-__device__ __forceinline__ void block_acc_init(BlockAcc& b)
-{
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < 3; ++i) b.pairs[i] = b.candidates[i] = 0;
-        for (int i = 0; i < 5; ++i) b.accepted[i] = b.created[i] = 0;
-        b.dE = 0.0;
-        b.status = 0;
-    }
-}
-
-__device__ __forceinline__ void block_acc_flush(const BlockAcc& b, DevStats* st)
-{
-    if (threadIdx.x != 0) return;
-    for (int i = 0; i < 3; ++i) {
-        if (b.pairs[i]) atomicAdd(&st->pairs[i], b.pairs[i]);
-        if (b.candidates[i]) atomicAdd(&st->candidates[i], b.candidates[i]);
-    }
-    for (int i = 0; i < 5; ++i) {
-        if (b.accepted[i]) atomicAdd(&st->accepted[i], b.accepted[i]);
-        if (b.created[i]) atomicAdd(&st->created[i], b.created[i]);
-    }
-    if (b.dE != 0.0) atomicAdd(&st->energy_change, b.dE);
-    if (b.status) atomicOr(&st->status, b.status);
 }
 
 // Candidate queues and per-call cell state of the batched path.
@@ -2024,18 +2091,6 @@ __device__ __forceinline__ CellRec fused_rec(const FusedWarp& w, int b, int g)
     return c;
 }
 
-// A thread's counters to the block's.
-__device__ __forceinline__ void add_rare(const Acc& acc, BlockAcc& b)
-{
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        if (acc.accepted[i]) atomicAdd(&b.accepted[i], (unsigned long long)acc.accepted[i]);
-        if (acc.created[i]) atomicAdd(&b.created[i], (unsigned long long)acc.created[i]);
-    }
-    if (acc.dE != 0.0) atomicAdd(&b.dE, acc.dE);
-    if (acc.status) atomicOr(&b.status, acc.status);
-}
-
 __device__ __forceinline__ void fused_event(FusedWarp& w, int b, int g, float rad, float wcre)
 {
     if (rad != 0.f) atomicAdd(&w.ev[b][g].x, rad);
@@ -2794,9 +2849,9 @@ int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_sp
         if (e != cudaSuccess) return cuda_fail(e, "pcc_collide: launch");
         if (run[g]) {
             if (precision == PCC_FP64_PLAIN) {
-                if (g == kGroupEm) collide_plain_kernel<kGroupEm><<<cells->n_cells, 128, 0, st>>>(a);
-                else if (g == kGroupEp) collide_plain_kernel<kGroupEp><<<cells->n_cells, 128, 0, st>>>(a);
-                else collide_plain_kernel<kGroupPh><<<cells->n_cells, 128, 0, st>>>(a);
+                if (g == kGroupEm) collide_plain_kernel<kGroupEm><<<cells->n_cells, kPlainThreads, 0, st>>>(a);
+                else if (g == kGroupEp) collide_plain_kernel<kGroupEp><<<cells->n_cells, kPlainThreads, 0, st>>>(a);
+                else collide_plain_kernel<kGroupPh><<<cells->n_cells, kPlainThreads, 0, st>>>(a);
                 note_launches(1);
             } else {
                 if (g == kGroupEm) e = launch_batched<kGroupEm>(ctx, a, stage, st);
