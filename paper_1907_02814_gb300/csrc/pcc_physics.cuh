@@ -47,22 +47,17 @@ __device__ inline double lambert_w0_neg(double z)
     return w;
 }
 
-// sum_{n>=2} n^-s, summed downward to n = 2000 plus the Euler-Maclaurin tail.
-__host__ __device__ inline double zeta_tail(double s)
-{
-    double acc = 0.0;
-    for (int n = 2000; n >= 2; --n) acc += exp(-s * log((double)n));
-    const double N = 2000.0;
-    return acc + exp((1.0 - s) * log(N)) / (s - 1.0) - 0.5 * exp(-s * log(N)) + s / 12.0 * exp((-s - 1.0) * log(N));
-}
-
 // Coulomb correction: a^2 [1/(1+a^2) + sum_{n=0}^{3} (-a^2)^n (zeta(2n+3) - 1)].
+// The values of zeta(3), zeta(5), zeta(7) and zeta(9) less one are mathematical
+// constants; summed from the series they took 12 ms of one thread.
 __host__ __device__ inline double coulomb_fc(int Z)
 {
+    const double zeta1[4] = {0.20205690315959428540, 0.03692775514336992633, 0.00834927738192282684,
+                             0.00200839282608221442};
     const double a2 = (kAlpha * Z) * (kAlpha * Z);
     double s = 0.0, p = 1.0;
     for (int n = 0; n < 4; ++n) {
-        s += p * zeta_tail(2.0 * n + 3.0);
+        s += p * zeta1[n];
         p *= -a2;
     }
     return a2 * (1.0 / (1.0 + a2) + s);
@@ -108,23 +103,103 @@ __device__ inline Screen screen_from_material(const pcc_material& m)
 
 // ---- Sec. II.B -------------------------------------------------------------
 
-// Eq. (deriv_I1).
-__device__ __forceinline__ double yukawa_I1(double d, double L)
+// atan x and ln(1 + x) by their Taylor series for |x| <= 1/8 and 0 <= x <= 1/64
+// (ten terms: the first dropped is below 2^-60 of the sum).
+__device__ __forceinline__ double atan_small(double x)
 {
-    const double L2 = L * L;
-    return L * d * (atan(L * d) - atan(L)) - 0.5 * L2 * (1.0 - d) * (1.0 - d) / (1.0 + L2) +
-           0.5 * log((1.0 + L2) / (1.0 + L2 * d * d));
+    const double s = x * x;
+    double t = -1.0 / 19.0;
+    t = t * s + 1.0 / 17.0;
+    t = t * s - 1.0 / 15.0;
+    t = t * s + 1.0 / 13.0;
+    t = t * s - 1.0 / 11.0;
+    t = t * s + 1.0 / 9.0;
+    t = t * s - 1.0 / 7.0;
+    t = t * s + 1.0 / 5.0;
+    t = t * s - 1.0 / 3.0;
+    return x + x * s * t;
+}
+__device__ __forceinline__ double log1p_small(double x)
+{
+    double t = -1.0 / 10.0;
+    t = t * x + 1.0 / 9.0;
+    t = t * x - 1.0 / 8.0;
+    t = t * x + 1.0 / 7.0;
+    t = t * x - 1.0 / 6.0;
+    t = t * x + 1.0 / 5.0;
+    t = t * x - 1.0 / 4.0;
+    t = t * x + 1.0 / 3.0;
+    t = t * x - 1.0 / 2.0;
+    return x + x * x * t;
 }
 
-// Eq. (deriv_I2).
-__device__ __forceinline__ double yukawa_I2(double d, double L)
+// What I1 and I2 of the reduced potential need of the length L alone.
+struct YukawaL {
+    double L, iL, L2, i1L2, rho, atanL, ln1L2, l1pi;   // 1/L, 1/(1+L^2), L^2/(1+L^2), atan L, ln(1+L^2), ln(1+L^-2)
+};
+__device__ inline YukawaL yukawa_length(double L)
 {
-    const double L2 = L * L, d2 = d * d;
-    const double t = 4.0 * L2 * L * d2 * d * (atan(L * d) - atan(L)) +
-                     (1.0 + 3.0 * L2 * d2) * log((1.0 + L2) / (1.0 + L2 * d2)) +
-                     6.0 * L2 * L2 * d2 / (1.0 + L2) * log(d) +
-                     L2 * (d - 1.0) * (d + 1.0 - 4.0 * L2 * d2) / (1.0 + L2);
-    return 0.5 * t;
+    YukawaL y;
+    y.L = L;
+    y.iL = 1.0 / L;
+    y.L2 = L * L;
+    y.i1L2 = 1.0 / (1.0 + y.L2);
+    y.rho = y.L2 * y.i1L2;
+    y.atanL = atan(L);
+    y.ln1L2 = log1p(y.L2);
+    y.l1pi = log1p(1.0 / y.L2);
+    return y;
+}
+
+// What they need of delta alone (shared by all materials): omd = 1 - delta, and
+// 1/delta, ln delta.
+struct YukawaD {
+    double d, omd, inv, ln;
+};
+
+// Eqs. (deriv_I1) and (deriv_I2) for u = L delta, in one of three forms that
+// form no difference of large terms: up to u = 1/8 and from u = 8 series take the
+// place of the logarithm, arc tangent and division.  (The printed form of I2
+// cancels terms of size u^2 ln L down to O(1) and takes two arc tangents and
+// three logarithms.)
+__device__ __forceinline__ void yukawa_I12(const YukawaL& y, const YukawaD& g, double& I1, double& I2)
+{
+    const double u = y.L * g.d, u2 = u * u;
+    const double q = y.rho * g.omd;          // rho (1 - d)
+    double lnr, A;                            // ln((1+L^2)/(1+u^2)), atan L - atan u
+    if (u > 8.0) {
+        const double iu = g.inv * y.iL, s = iu * iu, h = 1.0 / (1.0 + y.L * u);
+        const double z = g.omd * y.L * h;
+        const double l = y.l1pi - log1p_small(s);
+        A = atan_small(z);
+        lnr = l - 2.0 * g.ln;
+        // z - atan z from its series, without the cancellation
+        const double z2 = z * z;
+        double t = 1.0 / 21.0;
+        t = 1.0 / 19.0 - t * z2;
+        t = 1.0 / 17.0 - t * z2;
+        t = 1.0 / 15.0 - t * z2;
+        t = 1.0 / 13.0 - t * z2;
+        t = 1.0 / 11.0 - t * z2;
+        t = 1.0 / 9.0 - t * z2;
+        t = 1.0 / 7.0 - t * z2;
+        t = 1.0 / 5.0 - t * z2;
+        t = 1.0 / 3.0 - t * z2;
+        const double gz = t * z2 * z;
+        I2 = 0.5 * (-2.0 * g.ln - 6.0 * g.ln * u2 * y.i1L2 + (1.0 + 3.0 * u2) * l + 4.0 * u2 * u * gz +
+                    4.0 * g.omd * u2 * (h - y.i1L2) - q * (1.0 + g.d));
+    } else {
+        if (u <= 0.125) {
+            lnr = y.ln1L2 - log1p_small(u2);
+            A = y.atanL - atan_small(u);
+        } else {
+            const double f = 1.0 + u2, h = 1.0 + y.L * u, inv = 1.0 / (f * h);
+            lnr = log1p(y.L2 * g.omd * (1.0 + g.d) * (h * inv));
+            A = atan(y.L * g.omd * (f * inv));
+        }
+        I2 = 0.5 * (-4.0 * u2 * u * A + (1.0 + 3.0 * u2) * lnr + 6.0 * g.ln * u2 * y.rho + q * (4.0 * u2 - 1.0 - g.d));
+    }
+    I1 = -u * A - 0.5 * q * g.omd + 0.5 * lnr;
 }
 
 // g of Eq. (cs_br_nr).
@@ -172,51 +247,7 @@ __device__ inline double dsdk_nonrel(const Screen& s, double g1, double k, int p
     return born * (b1 / b2) * expm1(-a / b1) / expm1(-a / b2);
 }
 
-// delta of Eq. (csre): the minimum momentum transfer k / (2 gamma1 gamma2).
-__device__ __forceinline__ double brems_delta(double g1, double k) { return k / (2.0 * g1 * (g1 - k)); }
-
-// Eq. (csre) with fc = 0, Eq. (csur) with fc = f_C, for the screening
-// functions I1, I2 at delta = brems_delta(g1, k).
-__device__ inline double dsdk_relativistic_I(const Screen& s, double g1, double k, double fc, double I1, double I2)
-{
-    if (!(k > 0.0 && k < g1 - 1.0)) return 0.0;
-    const double eps = (g1 - k) / g1;
-    const double v = 4.0 * s.Z * s.Z * kRe * kRe * kAlpha / k *
-                     ((1.0 + eps * eps) * (I1 + 1.0 - fc) - (2.0 / 3.0) * eps * (I2 + 5.0 / 6.0 - fc));
-    return fmax(v, 0.0);
-}
-
-// The same with the reduced single-Yukawa potential at L = L_R.
-__device__ inline double dsdk_relativistic(const Screen& s, double g1, double k, double fc)
-{
-    const double d = brems_delta(g1, k);
-    return dsdk_relativistic_I(s, g1, k, fc, yukawa_I1(d, s.LR), yukawa_I2(d, s.LR));
-}
-
-__device__ __forceinline__ double dsdk_brems(const Screen& s, double g1, double k, int printed)
-{
-    if (g1 <= 2.0) return dsdk_nonrel(s, g1, k, printed);
-    return dsdk_relativistic(s, g1, k, g1 <= 100.0 ? 0.0 : s.fC);
-}
-
 // ---- Sec. II.C-D -----------------------------------------------------------
-
-// Eq. (dsdkbh) for the screening functions I1, I2 at delta = k / (2 gamma+ gamma-).
-__device__ inline double dsdg_bethe_heitler_I(const Screen& s, double k, double gp, double I1, double I2)
-{
-    const double gm = k - gp;
-    if (!(gp > 1.0 && gm > 1.0)) return 0.0;
-    const double v = 4.0 * s.Z * s.Z * kRe * kRe * kAlpha / (k * k * k) *
-                     ((gp * gp + gm * gm) * (I1 + 1.0) + (2.0 / 3.0) * gp * gm * (I2 + 5.0 / 6.0));
-    return fmax(v, 0.0);
-}
-
-// The same with the reduced single-Yukawa potential at L = L_R.
-__device__ inline double dsdg_bethe_heitler(const Screen& s, double k, double gp)
-{
-    const double d = k / (2.0 * gp * (k - gp));
-    return dsdg_bethe_heitler_I(s, k, gp, yukawa_I1(d, s.LR), yukawa_I2(d, s.LR));
-}
 
 // Gryaznykh fit of the total Trident cross section, zero below gamma1 = 3.
 template <typename T>
