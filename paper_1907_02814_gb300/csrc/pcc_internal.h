@@ -40,6 +40,10 @@ struct pcc_ctx {
     // pcc_bin: pinned copy of the totals and the event of its arrival
     void* bin_host = nullptr;
     cudaEvent_t bin_event = nullptr;
+    // quadrature of the expected-emission operator, for em_quad nodes
+    int em_quad = 0;
+    std::vector<float4> em_node;
+    std::vector<float2> em_node2;
     // cell work lists of the batched collision kernels (3 groups + class counters)
     int* lists = nullptr;
     int lists_cells = 0;

@@ -42,7 +42,8 @@ __device__ inline double lambert_w0_neg(double z)
         if (w1 == 0.0) break;
         const double step = f / (ew * w1 - 0.5 * (w + 2.0) * f / w1);
         w -= step;
-        if (fabs(step) <= 1e-16 * (1.0 + fabs(w))) break;
+        // the iteration is cubic: the next step would be below the last bit
+        if (fabs(step) <= 1e-9 * (1.0 + fabs(w))) break;
     }
     return w;
 }

@@ -53,8 +53,8 @@ def test_tables_against_the_oracle(orc, rows, cols, nodes, kw):
     mats = [(29, 5.0, 8.5e28, 100.0), (79, 30.0, 5.9e28, 1000.0), (13, 0.0, 6e28, 10.0), (1, 1.0, 1e25, 10.0)]
     mats += [(73, float(z), 5.55e28, 10.0 ** (1 + z / 20)) for z in range(1, 7)]      # ten: two chunks
     scr = orc.screening(orc.material(29, 2.0, 1e28, 100.0)).as_dict()
-    for off in (1e-8, 1e-3):         # Thomas-Fermi lengths stretched to nearly the Debye length
-        mats.append((29, 2.0, 1e28, 100.0, scr["LD"] / scr["LTF"] * (1.0 + off)))
+    for off in (1e-8, 1e-3):         # Debye lengths shrunk to nearly the Thomas-Fermi length
+        mats.append((29, 2.0, 1e28, 100.0, 1.0, scr["LTF"] / scr["LD"] * (1.0 + off)))
     ctx = pcc.Context(0)
     ctx.tables_build([pcc.material(*m) for m in mats], pcc.table_spec(n_rows=rows, n_cols=cols, quad_nodes=nodes, **kw))
     got = ctx.tables_read()
