@@ -84,6 +84,7 @@ __device__ __forceinline__ unsigned near_peers(int c)
 __global__ void bin_count_kernel(const int* __restrict__ cell, int n, int n_cells, int* __restrict__ counts,
                                  DevStats* st)
 {
+    pdl_begin();
     const int c = valid_cell(cell, blockIdx.x * blockDim.x + threadIdx.x, n, n_cells, st);
     const unsigned peers = near_peers(c);
     const int leader = __ffs(peers) - 1;
@@ -96,6 +97,7 @@ __global__ void bin_count_kernel(const int* __restrict__ cell, int n, int n_cell
 __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) bin_count_local_kernel(const int* __restrict__ cell, int n, int n_cells,
                                                                            int* __restrict__ counts, DevStats* st)
 {
+    pdl_begin();
     extern __shared__ int h[];
     const int lo = (int)((long long)n * blockIdx.x / gridDim.x), hi = (int)((long long)n * (blockIdx.x + 1) / gridDim.x);
     for (int c = threadIdx.x; c < n_cells; c += blockDim.x) h[c] = 0;
@@ -125,6 +127,7 @@ struct BlockSums {
 __global__ void __launch_bounds__(kScanBlock) region_sums_kernel(const int* __restrict__ counts, int n, int slack_abs,
                                                                  double slack_rel, BlockSums* __restrict__ sums)
 {
+    pdl_begin();
     __shared__ long long s[32];
     __shared__ int sp[32], sm[32];
     const int i = blockIdx.x * kScanBlock + threadIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -169,6 +172,7 @@ __global__ void __launch_bounds__(kScanBlock) region_offsets_kernel(const BlockS
                                                                     int* __restrict__ cursor, BinTotals* __restrict__ totals,
                                                                     SortLists L)
 {
+    pdl_begin();
     __shared__ long long sl[32];
     __shared__ int sp[32], sm[32], n_class[kSortClasses], at[kSortClasses];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -276,6 +280,7 @@ __device__ __forceinline__ void store_record(const MRec& out, int dst, const Tmp
 __global__ void bin_scatter_kernel(Rec in, const int* __restrict__ cell, int n, int n_cells, int* __restrict__ cursor,
                                    TmpRec* __restrict__ tmp, BinLimits lim)
 {
+    pdl_begin();
     if (lim.exceeded()) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int c = valid_cell(cell, i, n, n_cells, nullptr);
@@ -297,6 +302,7 @@ __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) bin_scatter_local
                                                                              int n_cells, int* __restrict__ cursor,
                                                                              TmpRec* __restrict__ tmp, BinLimits lim)
 {
+    pdl_begin();
     extern __shared__ int h[];
     if (lim.exceeded()) return;
     constexpr int kTile = kTileItems * kLocalThreads;
@@ -618,6 +624,7 @@ __global__ void __launch_bounds__(32 * kSortWarps, 12) sort_warp_kernel(const in
                                                                         const TmpRec* __restrict__ tmp, MRec out,
                                                                         BinLimits lim)
 {
+    pdl_begin();
     constexpr unsigned kFull = 0xffffffffu;
     __shared__ SortSmem<1, kSortWarpCap / 32> S[kSortWarps];
     const int c = blockIdx.x * kSortWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -655,6 +662,7 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 8 : 32 / ITEMS) sort_block_ke
                                                             const int* __restrict__ count, const TmpRec* __restrict__ tmp,
                                                             MRec out, BinLimits lim)
 {
+    pdl_begin();
     extern __shared__ __align__(16) unsigned char sort_smem[];
     auto& S = *reinterpret_cast<SortSmem<W, ITEMS>*>(sort_smem);
     if (lim.exceeded()) return;
@@ -669,6 +677,7 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 8 : 32 / ITEMS) sort_block_ke
 // ---- commit of appended secondaries: order by pid, then make live
 __global__ void commit_kernel(SpeciesView sp, int n_cells)
 {
+    pdl_begin();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c < n_cells) commit_cell(sp, c);
 }
@@ -677,6 +686,7 @@ __global__ void commit_kernel(SpeciesView sp, int n_cells)
 template <bool PHOTON>
 __global__ void __launch_bounds__(256, 4) totals_kernel(const pcc_species sp, int n_cells, double* __restrict__ partial)
 {
+    pdl_begin();
     __shared__ double sh[3][32];
     const int nw = blockDim.x >> 5;
     TotalsAcc acc;
@@ -684,7 +694,8 @@ __global__ void __launch_bounds__(256, 4) totals_kernel(const pcc_species sp, in
     totals_block_out(acc, sh, partial);
 }
 
-__global__ void totals_final_kernel(const double* partial, int nb, double* out) { totals_reduce(partial, nb, out); }
+__global__ void totals_final_kernel(const double* partial, int nb, double* out) {
+    pdl_begin(); totals_reduce(partial, nb, out); }
 
 }  // namespace pcc
 
@@ -714,7 +725,7 @@ static void launch_sort(pcc_ctx* ctx, int cls, const pcc_species* out, const int
 {
     constexpr int smem = (int)sizeof(SortSmem<W, ITEMS>);
     constexpr int per_sm = std::min(2048 / (32 * W), 227 * 1024 / (smem + 1024));
-    sort_block_kernel<W, ITEMS><<<per_sm * std::max(ctx->num_sms, 1), 32 * W, smem, st>>>(
+    launch_pdl(sort_block_kernel<W, ITEMS>, per_sm * std::max(ctx->num_sms, 1), 32 * W, smem, st, 
         out->cell_start, out->cell_count, first, L.list[cls], L.count + cls, tmp, ro, lim);
     note_launches(1);
 }
@@ -776,12 +787,12 @@ extern "C" int pcc_bin(pcc_ctx* ctx, const pcc_particles* in, int n_cells, pcc_s
     cudaError_t e = cudaMemsetAsync(counts, 0, ((size_t)n_cells + kSortClasses) * sizeof(int), st);
     if (e != cudaSuccess) return cuda_fail(e, "pcc_bin: memset");
     if (n > 0) {
-        if (local) bin_count_local_kernel<<<blocks, kLocalThreads, local_smem, st>>>(in->cell, n, n_cells, counts, ctx->stats);
-        else bin_count_kernel<<<(n + 255) / 256, 256, 0, st>>>(in->cell, n, n_cells, counts, ctx->stats);
+        if (local) launch_pdl(bin_count_local_kernel, blocks, kLocalThreads, local_smem, st, in->cell, n, n_cells, counts, ctx->stats);
+        else launch_pdl(bin_count_kernel, (n + 255) / 256, 256, 0, st, in->cell, n, n_cells, counts, ctx->stats);
         note_launches(1);
     }
-    region_sums_kernel<<<nb, kScanBlock, 0, st>>>(counts, n_cells, slack_abs, slack_rel, sums);
-    region_offsets_kernel<<<nb, kScanBlock, 0, st>>>(sums, nb, counts, n_cells, slack_abs, slack_rel, out->cell_start,
+    launch_pdl(region_sums_kernel, nb, kScanBlock, 0, st, counts, n_cells, slack_abs, slack_rel, sums);
+    launch_pdl(region_offsets_kernel, nb, kScanBlock, 0, st, sums, nb, counts, n_cells, slack_abs, slack_rel, out->cell_start,
                                                      out->cell_count, out->cell_added, first, cursor, tot, L);
     note_launches(2);
     // the host learns the totals while the records move: the kernels below
@@ -794,13 +805,13 @@ extern "C" int pcc_bin(pcc_ctx* ctx, const pcc_particles* in, int n_cells, pcc_s
         const BinLimits lim{tot, (long long)out->capacity};
         const Rec rin{in->ux, in->uy, in->uz, in->w, out->x ? in->x : nullptr, in->pid};
         const MRec ro{out->ux, out->uy, out->uz, out->w, out->x, out->pid};
-        if (local) bin_scatter_local_kernel<<<blocks, kLocalThreads, local_smem, st>>>(rin, in->cell, n, n_cells, cursor, tmp, lim);
-        else bin_scatter_kernel<<<(n + 255) / 256, 256, 0, st>>>(rin, in->cell, n, n_cells, cursor, tmp, lim);
+        if (local) launch_pdl(bin_scatter_local_kernel, blocks, kLocalThreads, local_smem, st, rin, in->cell, n, n_cells, cursor, tmp, lim);
+        else launch_pdl(bin_scatter_kernel, (n + 255) / 256, 256, 0, st, rin, in->cell, n, n_cells, cursor, tmp, lim);
         // the fullest cells first: their blocks run longest
         if (n > kSortCap1) launch_sort<16, 32>(ctx, 2, out, first, L, tmp, ro, lim, st);
         if (n > kSortCap0) launch_sort<16, 16>(ctx, 1, out, first, L, tmp, ro, lim, st);
         if (n > kSortWarpCap) launch_sort<4, 16>(ctx, 0, out, first, L, tmp, ro, lim, st);
-        sort_warp_kernel<<<(n_cells + kSortWarps - 1) / kSortWarps, 32 * kSortWarps, 0, st>>>(
+        launch_pdl(sort_warp_kernel, (n_cells + kSortWarps - 1) / kSortWarps, 32 * kSortWarps, 0, st, 
             out->cell_start, out->cell_count, first, n_cells, tmp, ro, lim);
         note_launches(2);
     }
@@ -825,7 +836,7 @@ extern "C" int pcc_append_secondaries(pcc_ctx* ctx, int n_cells, pcc_species* sp
         set_error("pcc_append_secondaries: invalid argument");
         return PCC_E_INVALID;
     }
-    commit_kernel<<<(n_cells + 255) / 256, 256, 0, (cudaStream_t)stream>>>(view_of(*sp), n_cells);
+    launch_pdl(commit_kernel, (n_cells + 255) / 256, 256, 0, (cudaStream_t)stream, view_of(*sp), n_cells);
     note_launches(1);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PCC_OK : cuda_fail(e, "pcc_append_secondaries");
@@ -841,9 +852,9 @@ extern "C" int pcc_totals(pcc_ctx* ctx, int n_cells, const pcc_species* sp, int 
     if (rc) return rc;
     double* partial = (double*)ctx->scratch;
     cudaStream_t st = (cudaStream_t)stream;
-    if (is_photon) totals_kernel<true><<<blocks, 256, 0, st>>>(*sp, n_cells, partial);
-    else totals_kernel<false><<<blocks, 256, 0, st>>>(*sp, n_cells, partial);
-    totals_final_kernel<<<1, 96, 0, st>>>(partial, blocks, out);
+    if (is_photon) launch_pdl(totals_kernel<true>, blocks, 256, 0, st, *sp, n_cells, partial);
+    else launch_pdl(totals_kernel<false>, blocks, 256, 0, st, *sp, n_cells, partial);
+    launch_pdl(totals_final_kernel, 1, 96, 0, st, partial, blocks, out);
     note_launches(2);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PCC_OK : cuda_fail(e, "pcc_totals");

@@ -857,6 +857,7 @@ __device__ void plain_bh_cell(const CtaGroup& grp, PlainShared& S, const StepArg
 template <int GROUP>
 __global__ void __launch_bounds__(kPlainThreads, 8) collide_plain_kernel(const __grid_constant__ StepArgs a)
 {
+    pdl_begin();
     __shared__ PlainShared S;
     const CtaGroup grp{S.scratch, S.red};
     if (GROUP == kGroupPh) plain_bh_cell(grp, S, a, blockIdx.x);
@@ -921,6 +922,7 @@ struct ClassSort {
     const int* cnt_t;      // ion counts
     int n_cells;
     unsigned run;          // bit g: group g is sorted
+    int* counters;         // the groups' queue counters
     unsigned* serial;      // collide calls so far (stamps the per-cell ion summaries)
 };
 
@@ -934,6 +936,7 @@ struct ClassSort {
 __global__ void class_hist_kernel(const __grid_constant__ ClassSort S)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) *S.serial += 1u;   // a new call: earlier summaries go stale
+    if (blockIdx.x == 0 && threadIdx.x < 12) S.counters[threadIdx.x] = 0;
     __shared__ int h[3][kClasses];
     for (int i = threadIdx.x; i < 3 * kClasses; i += blockDim.x) (&h[0][0])[i] = 0;
     __syncthreads();
@@ -2522,7 +2525,7 @@ static int persistent_grid(pcc_ctx* ctx, const void* fn, int smem, int want_per_
 //   [6n) cells with events                   [7n) listed flags
 //   [8n, 10n) ledger contributions (float2)  [R, R + 8n) cell records (int4 pairs,
 //   R = 10n rounded up to 4 ints)           [R + 8n) class histograms and cursors,
-//   then three counters (flat queue, N_p < N_t cells, cells with events), then
+//   then the counters (see counters_of), then
 //   the per-block class counts of the three groups.
 // Flags and contributions start at zero and are cleared by the finalize kernel.
 static size_t rec_off(size_t n) { return (10 * n + 3) & ~(size_t)3; }
@@ -2531,7 +2534,7 @@ static size_t hist_off(size_t n) { return rec_off(n) + 8 * n; }
 static size_t ionsum_off(size_t n)
 {
     const size_t nblk = (n + kClassBlock - 1) / kClassBlock;
-    return (hist_off(n) + 6 * kClasses + 8 + 3 * kClasses * nblk + 3) & ~(size_t)3;
+    return (hist_off(n) + 6 * kClasses + 16 + 3 * kClasses * nblk + 3) & ~(size_t)3;
 }
 
 static int ensure_lists(pcc_ctx* ctx, int n_cells)
@@ -2577,26 +2580,28 @@ static CellList list_of(pcc_ctx* ctx, int group)
     L.hist = ctx->lists + hist_off(n) + (size_t)(2 * group) * kClasses;
     L.cursor = L.hist + kClasses;
     L.nblk = (int)((n + kClassBlock - 1) / kClassBlock);
-    L.bh = ctx->lists + hist_off(n) + 6 * kClasses + 8 + (size_t)group * kClasses * L.nblk;
+    L.bh = ctx->lists + hist_off(n) + 6 * kClasses + 16 + (size_t)group * kClasses * L.nblk;
     for (int i = 0; i < 4; ++i) L.thr[i] = ctx->scan_thr[group][i];
     return L;
 }
 
+// Counters: [4 g ..] of group g (flat queue, N_p < N_t cells, cells with events),
+// cleared by the class histogram of each call; then the call serial (never cleared).
+constexpr int kCounters = 16, kSerial = 12;
 static int* counters_of(pcc_ctx* ctx) { return ctx->lists + hist_off(ctx->lists_cells) + 6 * kClasses; }
 
-// counters: [0..2] cleared per group; [4] the call serial (never cleared)
 static IonCache ion_cache_of(pcc_ctx* ctx)
 {
     IonCache C;
     C.sum = reinterpret_cast<float4*>(ctx->lists + ionsum_off(ctx->lists_cells));
-    C.serial = reinterpret_cast<const unsigned*>(counters_of(ctx) + 4);
+    C.serial = reinterpret_cast<const unsigned*>(counters_of(ctx) + kSerial);
     return C;
 }
 
-static Queue queue_of(pcc_ctx* ctx)
+static Queue queue_of(pcc_ctx* ctx, int group)
 {
     const size_t n = ctx->lists_cells;
-    int* c = counters_of(ctx);
+    int* c = counters_of(ctx) + 4 * group;
     Queue Q;
     Q.flat = (uint2*)ctx->queue_a;
     Q.cap_flat = (uint32_t)std::min<size_t>(ctx->queue_a_cap, 0xFFFFFFFFu);
@@ -2626,10 +2631,8 @@ static void launch_scan(pcc_ctx* ctx, const StepArgs& a, const CellList& L, cons
 template <int GROUP>
 static cudaError_t launch_batched(pcc_ctx* ctx, const StepArgs& a, int stage, cudaStream_t st)
 {
-    cudaError_t e = cudaMemsetAsync(counters_of(ctx), 0, 3 * sizeof(int), st);
-    if (e != cudaSuccess) return e;
     const CellList L = list_of(ctx, GROUP);
-    const Queue Q = queue_of(ctx);
+    const Queue Q = queue_of(ctx, GROUP);
     switch (ctx->minb) {
     case 2: launch_scan<GROUP, 2>(ctx, a, L, Q, st); break;
     case 3: launch_scan<GROUP, 3>(ctx, a, L, Q, st); break;
@@ -2657,7 +2660,8 @@ static void launch_class_sort(pcc_ctx* ctx, const StepArgs& a, unsigned run, cud
     S.cnt_t = a.ion.count;
     S.n_cells = a.n_cells;
     S.run = run;
-    S.serial = reinterpret_cast<unsigned*>(counters_of(ctx) + 4);
+    S.counters = counters_of(ctx);
+    S.serial = reinterpret_cast<unsigned*>(counters_of(ctx) + kSerial);
     const int nblk = S.L[0].nblk;
     class_hist_kernel<<<nblk, kClassBlock, 0, st>>>(S);
     const size_t off_smem = (size_t)kClasses * nblk * sizeof(int);
@@ -2849,9 +2853,9 @@ int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_sp
         if (e != cudaSuccess) return cuda_fail(e, "pcc_collide: launch");
         if (run[g]) {
             if (precision == PCC_FP64_PLAIN) {
-                if (g == kGroupEm) collide_plain_kernel<kGroupEm><<<cells->n_cells, kPlainThreads, 0, st>>>(a);
-                else if (g == kGroupEp) collide_plain_kernel<kGroupEp><<<cells->n_cells, kPlainThreads, 0, st>>>(a);
-                else collide_plain_kernel<kGroupPh><<<cells->n_cells, kPlainThreads, 0, st>>>(a);
+                if (g == kGroupEm) launch_pdl(collide_plain_kernel<kGroupEm>, cells->n_cells, kPlainThreads, 0, st, a);
+                else if (g == kGroupEp) launch_pdl(collide_plain_kernel<kGroupEp>, cells->n_cells, kPlainThreads, 0, st, a);
+                else launch_pdl(collide_plain_kernel<kGroupPh>, cells->n_cells, kPlainThreads, 0, st, a);
                 note_launches(1);
             } else {
                 if (g == kGroupEm) e = launch_batched<kGroupEm>(ctx, a, stage, st);

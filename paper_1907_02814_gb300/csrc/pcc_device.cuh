@@ -19,6 +19,16 @@ constexpr double kEps0 = 8.8541878128e-12;       // vacuum permittivity [F/m]
 constexpr double kQe = 1.602176634e-19;          // elementary charge [C]
 constexpr double kPi = 3.14159265358979323846;
 
+// First statement of a kernel launched by launch_pdl, on every thread: lets the
+// kernel after it come in as blocks leave, then waits for the one before it to
+// complete, its writes included.  Since every kernel of a chain waits, all
+// earlier ones are complete too.
+__device__ __forceinline__ void pdl_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Random-stream tags: group | purpose << 4 | pass << 8 (Philox counter word 3).
 enum Group : uint32_t { kGroupEm = 0, kGroupEp = 1, kGroupPh = 2 };
 enum Purpose : uint32_t { kPerm = 0, kAccept = 1, kEvtBrems = 2, kEvtTri1 = 3, kEvtTri2 = 4, kEvtBH = 5,

@@ -81,6 +81,29 @@ int ensure_scratch(pcc_ctx* ctx, size_t bytes);
 void note_launches(unsigned long long n);
 unsigned long long launches_so_far();
 
+// Launch with programmatic stream serialization: the kernel's blocks may take
+// their places while the last blocks of the kernel before it still run, and wait
+// there (pdl_begin) until it is complete.  Used for the chains of short kernels
+// (binning of 60 small cells 44 -> 37 us, of a 1e5-cell step's species 1.41 -> 1.38
+// ms with its collide); the persistent kernels of the batched step, which
+// fill every SM to the end, lose by it (2^20 cells 1.145 -> 1.165 ms, 16 foil steps
+// 0.99 -> 1.05 ms) and are launched plainly.
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A&&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Table geometry passed to kernels by value.
 struct TableGeom {
     int n_rows, n_cols;
