@@ -880,9 +880,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)_
 struct CellList {
     int* list;       // [n_cells], cells by decreasing size class
     int* hist;       // [kClasses] cells per class
-    int* cursor;     // [kClasses] (unused)
-    int* bh;         // [kClasses][nblk] per-block class counts, then their offsets
-    int nblk;        // blocks of kClassBlock cells
+    int* cursor;     // [kClasses] next free entry per class while the list is filled
+    int* total;      // [kClasses] counts of the call, zero between calls
     int thr[4];      // scan lane groups: classes >= thr[0] a whole warp, [thr[1], thr[0]) 16 lanes,
                      // [thr[2], thr[1]) 8, [thr[3], thr[2]) 4, below 2 (pcc_set_scan_classes)
 };
@@ -900,7 +899,6 @@ constexpr int kFusedMinCells = 32;
 constexpr int kFusedCellsPerWarp = 5;
 constexpr int kFusedWarpsPerSM = 24;
 constexpr int kClassBlock = 1024;                 // cells per class-sort block
-constexpr int kClassSmemMax = 200 * 1024;         // offsets scanned in shared memory up to this size
 
 // Class of a cell with N_pair = max(N_p, N_t) pairs: with b the bit length
 // of N_pair, class 2(b - 1) for N_pair in [2^(b-1), 1.5 2^(b-1)) and
@@ -926,13 +924,14 @@ struct ClassSort {
     unsigned* serial;      // collide calls so far (stamps the per-cell ion summaries)
 };
 
-// Counting sort of the cells with both species by decreasing size class,
-// in three passes without global atomics: per-block class counts, their
-// exclusive scan (classes from the largest, blocks in order), and the
-// scatter with ranks from shared-memory counters.  The order within one
-// block's cells of one class follows the shared atomics and may differ from
-// run to run; no result depends on it, since every cell is processed
-// independently of where it sits in the list.
+// Counting sort of the cells with both species by decreasing size class, in
+// three passes: class counts, added up per block in shared memory and once per
+// class and block in global memory; where each class starts; and the scatter,
+// in which a block takes places for its cells of a class with one atomic.  The
+// order within a class may differ from run to run; no result depends on it,
+// since every cell is processed independently of where it sits in the list.
+// (Scanning 34 counts of every block, in one block per group, took longer than
+// the two passes over the cells: 24 us of a 2^20-cell step.)
 __global__ void class_hist_kernel(const __grid_constant__ ClassSort S)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) *S.serial += 1u;   // a new call: earlier summaries go stale
@@ -953,96 +952,51 @@ __global__ void class_hist_kernel(const __grid_constant__ ClassSort S)
     __syncthreads();
     for (int i = threadIdx.x; i < 3 * kClasses; i += blockDim.x) {
         const int g = i / kClasses, k = i - g * kClasses;
-        if (S.run >> g & 1u) S.L[g].bh[k * S.L[g].nblk + blockIdx.x] = h[g][k];
+        if (h[g][k]) atomicAdd(&S.L[g].total[k], h[g][k]);
     }
 }
 
-// One block per group: bh[k][b] -> offset of block b's cells of class k in
-// the list; hist[k] -> cells of class k.  The counts are staged in shared
-// memory when they fit (SMEM = true), else scanned in place in global memory.
-template <bool SMEM>
-__global__ void __launch_bounds__(1024) class_offsets_kernel(const __grid_constant__ ClassSort S)
+// One thread per group and class: cells of the class, and where it starts (after
+// all larger classes); the totals go back to zero.
+__global__ void class_offsets_kernel(const __grid_constant__ ClassSort S)
 {
-    extern __shared__ int sm[];
-    __shared__ int part[32];
-    if (!(S.run >> blockIdx.x & 1u)) return;
-    const CellList& L = S.L[blockIdx.x];
-    const int n = kClasses * L.nblk;
-    int* v = SMEM ? sm : L.bh;
-    if (SMEM)
-        for (int i = threadIdx.x; i < n; i += blockDim.x) sm[i] = L.bh[i];
-    __syncthreads();
-    // scan order: classes from the largest, blocks in order; thread t takes
-    // a contiguous chunk [i0, i1) of that order, entry (class k, block b)
-    // stepped without divisions
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int i0 = min((int)threadIdx.x * per, n), i1 = min(i0 + per, n);
-    const int k0 = kClasses - 1 - i0 / L.nblk, b0 = i0 - (kClasses - 1 - k0) * L.nblk;
-    int sum = 0;
-    for (int e = i0, k = k0, b = b0; e < i1; ++e) {
-        sum += v[k * L.nblk + b];
-        if (++b == L.nblk) { b = 0; --k; }
-    }
-    // exclusive scan of the thread sums: within each warp by shuffles, then
-    // over the warp totals
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) part[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        int x = lane < nw ? part[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += t;
-        }
-        part[lane] = x;
+    __shared__ int t[3][kClasses];
+    const int g = threadIdx.x / kClasses, k = threadIdx.x - g * kClasses;
+    if (g < 3) {
+        t[g][k] = S.L[g].total[k];
+        S.L[g].total[k] = 0;
     }
     __syncthreads();
-    int run = (wid ? part[wid - 1] : 0) + incl - sum;
-    for (int e = i0, k = k0, b = b0; e < i1; ++e) {
-        int& x = v[k * L.nblk + b];
-        const int c = x;
-        x = run;
-        run += c;
-        if (++b == L.nblk) { b = 0; --k; }
-    }
-    __syncthreads();
-    // class k occupies [offset of its block 0, offset of block 0 of class
-    // k - 1) of the list; class 0 ends at the total
-    if (threadIdx.x < kClasses) {
-        const int k = threadIdx.x;
-        const int end = k == 0 ? part[nw - 1] : v[(k - 1) * L.nblk];
-        L.hist[k] = end - v[k * L.nblk];
-    }
-    if (SMEM)
-        for (int i = threadIdx.x; i < n; i += blockDim.x) L.bh[i] = sm[i];
+    if (g >= 3) return;
+    int at = 0;
+    for (int q = k + 1; q < kClasses; ++q) at += t[g][q];
+    S.L[g].hist[k] = t[g][k];
+    S.L[g].cursor[k] = at;
 }
 
 __global__ void class_scatter_kernel(const __grid_constant__ ClassSort S)
 {
-    __shared__ int rank[3][kClasses];
-    for (int i = threadIdx.x; i < 3 * kClasses; i += blockDim.x) (&rank[0][0])[i] = 0;
+    __shared__ int h[3][kClasses];
+    for (int i = threadIdx.x; i < 3 * kClasses; i += blockDim.x) (&h[0][0])[i] = 0;
     __syncthreads();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < S.n_cells) {
-        const int nt = S.cnt_t[c];
+    int cls[3], rank[3];
+    const int nt = c < S.n_cells ? S.cnt_t[c] : 0;
 #pragma unroll
-        for (int g = 0; g < 3; ++g) {
-            if (!(S.run >> g & 1u) || nt <= 0) continue;
-            const int np = S.cnt_p[g][c];
-            if (np > 0) {
-                const int cls = size_class(np, nt);
-                const CellList& L = S.L[g];
-                L.list[L.bh[cls * L.nblk + blockIdx.x] + atomicAdd(&rank[g][cls], 1)] = c;
-            }
-        }
+    for (int g = 0; g < 3; ++g) {
+        const int np = nt > 0 && (S.run >> g & 1u) ? S.cnt_p[g][c] : 0;
+        cls[g] = np > 0 ? size_class(np, nt) : -1;
+        rank[g] = np > 0 ? atomicAdd(&h[g][cls[g]], 1) : 0;
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * kClasses; i += blockDim.x) {
+        const int g = i / kClasses, k = i - g * kClasses;
+        if (h[g][k]) h[g][k] = atomicAdd(&S.L[g].cursor[k], h[g][k]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int g = 0; g < 3; ++g)
+        if (cls[g] >= 0) S.L[g].list[h[g][cls[g]] + rank[g]] = c;
 }
 
 // Poll the mbarrier at smem address b for phase 0, at most `polls` times;
@@ -2525,16 +2479,16 @@ static int persistent_grid(pcc_ctx* ctx, const void* fn, int smem, int want_per_
 //   [6n) cells with events                   [7n) listed flags
 //   [8n, 10n) ledger contributions (float2)  [R, R + 8n) cell records (int4 pairs,
 //   R = 10n rounded up to 4 ints)           [R + 8n) class histograms and cursors,
-//   then the counters (see counters_of), then
-//   the per-block class counts of the three groups.
-// Flags and contributions start at zero and are cleared by the finalize kernel.
+//   then the counters (see counters_of), then the class totals of the three groups.
+// Flags and contributions start at zero and are cleared by the finalize kernel,
+// the class totals by the class offsets.
+constexpr int kCounters = 16, kSerial = 12;
 static size_t rec_off(size_t n) { return (10 * n + 3) & ~(size_t)3; }
 static size_t hist_off(size_t n) { return rec_off(n) + 8 * n; }
 // then, 16-byte aligned, the per-cell ion summaries (float4, see IonCache)
 static size_t ionsum_off(size_t n)
 {
-    const size_t nblk = (n + kClassBlock - 1) / kClassBlock;
-    return (hist_off(n) + 6 * kClasses + 16 + 3 * kClasses * nblk + 3) & ~(size_t)3;
+    return (hist_off(n) + 9 * kClasses + kCounters + 3) & ~(size_t)3;
 }
 
 static int ensure_lists(pcc_ctx* ctx, int n_cells)
@@ -2579,15 +2533,13 @@ static CellList list_of(pcc_ctx* ctx, int group)
     L.list = ctx->lists + (size_t)group * n;
     L.hist = ctx->lists + hist_off(n) + (size_t)(2 * group) * kClasses;
     L.cursor = L.hist + kClasses;
-    L.nblk = (int)((n + kClassBlock - 1) / kClassBlock);
-    L.bh = ctx->lists + hist_off(n) + 6 * kClasses + 16 + (size_t)group * kClasses * L.nblk;
+    L.total = ctx->lists + hist_off(n) + 6 * kClasses + kCounters + (size_t)group * kClasses;
     for (int i = 0; i < 4; ++i) L.thr[i] = ctx->scan_thr[group][i];
     return L;
 }
 
 // Counters: [4 g ..] of group g (flat queue, N_p < N_t cells, cells with events),
 // cleared by the class histogram of each call; then the call serial (never cleared).
-constexpr int kCounters = 16, kSerial = 12;
 static int* counters_of(pcc_ctx* ctx) { return ctx->lists + hist_off(ctx->lists_cells) + 6 * kClasses; }
 
 static IonCache ion_cache_of(pcc_ctx* ctx)
@@ -2662,11 +2614,9 @@ static void launch_class_sort(pcc_ctx* ctx, const StepArgs& a, unsigned run, cud
     S.run = run;
     S.counters = counters_of(ctx);
     S.serial = reinterpret_cast<unsigned*>(counters_of(ctx) + kSerial);
-    const int nblk = S.L[0].nblk;
+    const int nblk = (a.n_cells + kClassBlock - 1) / kClassBlock;
     class_hist_kernel<<<nblk, kClassBlock, 0, st>>>(S);
-    const size_t off_smem = (size_t)kClasses * nblk * sizeof(int);
-    if (off_smem <= (size_t)kClassSmemMax) class_offsets_kernel<true><<<3, 1024, off_smem, st>>>(S);
-    else class_offsets_kernel<false><<<3, 1024, 0, st>>>(S);
+    class_offsets_kernel<<<1, 128, 0, st>>>(S);
     class_scatter_kernel<<<nblk, kClassBlock, 0, st>>>(S);
     note_launches(3);
 }
@@ -2722,12 +2672,6 @@ int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em,
     if (!ctx || !cells || !em || !ep || !ph || !ion || cells->n_cells < 1) {
         set_error("pcc_collide: invalid argument");
         return PCC_E_INVALID;
-    }
-    if (!ctx->class_smem_ready) {   // per device, before any capture
-        if (cudaFuncSetAttribute(class_offsets_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kClassSmemMax) != cudaSuccess)
-            return cuda_fail(cudaGetLastError(), "pcc_collide: class sort shared memory");
-        ctx->class_smem_ready = true;
     }
     if (precision != PCC_FP32_BATCHED) return PCC_OK;
     const unsigned groups = (mask & 0x700u) ? (mask & 0x700u) : 0x700u;

@@ -59,7 +59,6 @@ struct pcc_ctx {
     // batched Cu workload; the autotuner may replace them.
     int scan_thr[3][4] = {{20, 20, 15, 2}, {12, 12, 6, 0}, {17, 17, 15, 13}};
     int blocks_per_sm = 0;         // persistent grid cap (0: as many as fit)
-    bool class_smem_ready = false; // large shared memory enabled for the class-sort offsets
     int wait_polls = pcc::kWaitPolls;   // bounded waits give up after this many polls (fault injection: 0)
     // resident blocks per SM of the persistent kernels, by (kernel, dynamic smem)
     struct Occ { const void* fn; int smem; int per_sm; };
