@@ -92,8 +92,8 @@ __global__ void bin_count_kernel(const int* __restrict__ cell, int n, int n_cell
 }
 
 // Few cells: a block counts a contiguous chunk of the input in shared memory
-// and adds a cell's count once.  2048 cells of 8192 shuffled particles took
-// 0.70 ms with a global atomic per particle.
+// and adds a cell's count once: 2048 cells of 8192 shuffled particles 0.70 -> 0.06
+// ms (a global atomic per particle before).
 __global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) bin_count_local_kernel(const int* __restrict__ cell, int n, int n_cells,
                                                                            int* __restrict__ counts, DevStats* st)
 {
@@ -162,8 +162,8 @@ __device__ __forceinline__ int sort_class(int count)
 }
 
 // Each block adds up the sums of the blocks before it and scans its own cells:
-// one thread that walked the block sums, and one atomic maximum per cell, were
-// a quarter of a small call before.
+// the atomic maximum of every cell alone took 64 us of a 1e5-cell binning, and
+// one thread walked the block sums.
 __global__ void __launch_bounds__(kScanBlock) region_offsets_kernel(const BlockSums* __restrict__ sums, int nb,
                                                                     const int* __restrict__ counts, int n, int slack_abs,
                                                                     double slack_rel, int* __restrict__ cell_start,
@@ -779,7 +779,7 @@ extern "C" int pcc_bin(pcc_ctx* ctx, const pcc_particles* in, int n_cells, pcc_s
 
     // Counting and handing out places in shared memory pays where a block's
     // chunk holds several particles for each counter: 2048 cells x 8192
-    // shuffled particles, count 0.70 -> 0.04 ms.
+    // shuffled particles, count 0.70 -> 0.06 ms, scatter 1.18 -> 0.37 ms.
     const int blocks = kLocalBlocks * std::max(ctx->num_sms, 1);
     const bool local = n_cells <= kLocalCells && n >= 4ll * n_cells * blocks;
     const size_t local_smem = (size_t)n_cells * sizeof(int);

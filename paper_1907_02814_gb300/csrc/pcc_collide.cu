@@ -1,11 +1,13 @@
 // The pairwise collision step of Sec. III.A for electron-ion (Bremsstrahlung
 // then Trident on each pair), positron-ion and photon-ion (Bethe-Heitler)
-// pairs.  One routine per cell, templated on the arithmetic type and on the
-// thread group that owns the cell:
+// pairs.
 //   plain   (FP64): one thread block per cell, grid = cells;
-//   batched (FP32): persistent grid, one warp per cell, cells strided over
-//                   warps, ln sigma rows staged in shared memory by a bulk
-//                   copy (cp.async.bulk + mbarrier).
+//   batched (FP32): up to five cells per resident warp, one kernel that takes a
+//                   warp's cells through everything; beyond, cells sorted by
+//                   size, a scan that queues the few pairs whose accept digits
+//                   pass a bound, and kernels that evaluate those, with the ln
+//                   sigma rows staged in shared memory by a bulk copy
+//                   (cp.async.bulk + mbarrier).
 #include <algorithm>
 
 #include "pcc_commit.cuh"
