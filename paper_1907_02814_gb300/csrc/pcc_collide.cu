@@ -480,8 +480,9 @@ __device__ __forceinline__ void ei_pair(const StepArgs* ap, const Tab<Real>& tb,
 // x <= coef B, and p <= x), or its energy, by a float bound with a margin, may lie
 // above the tables, or its momentum is not plainly finite, so that the status
 // bits come out as if every pair were evaluated.  A step of 16384 Au cells of 256
-// electrons, 64 ions and 64 photons takes 0.55 ms (3.59 ms with every pair
+// electrons, 64 ions and 64 photons takes 0.33 ms (3.59 ms with every pair
 // evaluated), bound by the latency of a block's phases.
+// Threads of a block at most (see plain_threads).
 constexpr int kPlainThreads = 128, kPlainWarps = kPlainThreads / 32;
 
 // Per-block counters, updated with shared atomics and added to the context's
@@ -559,7 +560,7 @@ __device__ __forceinline__ void plain_sums(const CtaGroup& grp, PlainShared& S, 
     const float w0 = I.w[c.t0];
     double sp = 0, st = 0, sf = 0;
     float wmin = w0, wmax = w0, u2m = 0.f, u2s = 0.f;
-    for (uint32_t s = threadIdx.x; s < Nt; s += kPlainThreads) {
+    for (uint32_t s = threadIdx.x; s < Nt; s += blockDim.x) {
         const int t = c.t0 + (int)s;
         const float wt = I.w[t], ux = I.ux[t], uy = I.uy[t], uz = I.uz[t];
         st += (double)wt;
@@ -571,13 +572,13 @@ __device__ __forceinline__ void plain_sums(const CtaGroup& grp, PlainShared& S, 
     }
     if (c.pr.caseA) {
 #pragma unroll 4
-        for (uint32_t s = threadIdx.x; s < Np; s += kPlainThreads) {
+        for (uint32_t s = threadIdx.x; s < Np; s += blockDim.x) {
             const float wp = P.w[c.p0 + (int)s];
             sp += (double)wp;
             sf += (double)fminf(wp, w0);
         }
     } else {
-        for (uint32_t s = threadIdx.x; s < Np; s += kPlainThreads) {
+        for (uint32_t s = threadIdx.x; s < Np; s += blockDim.x) {
             const float wp = P.w[c.p0 + (int)s];
             sp += (double)wp;
             sf += (double)fminf(wp, w0) * (double)((Nt - s + Np - 1) / Np);
@@ -603,7 +604,7 @@ __device__ __forceinline__ void plain_sums(const CtaGroup& grp, PlainShared& S, 
     __syncthreads();
     double n_p = 0, n_t = 0, n_pt = 0;
     float lo = S.lo[0], hi = S.hi[0], um = 0.f;
-    for (int k = 0; k < kPlainWarps; ++k) {
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
         n_p += S.sum[0][k];
         n_t += S.sum[1][k];
         n_pt += S.sum[2][k];
@@ -616,7 +617,7 @@ __device__ __forceinline__ void plain_sums(const CtaGroup& grp, PlainShared& S, 
     c.fac = um < 1e12f ? 1.0 + (double)fminf(ui / gi * 1.0001f, 1.f) : 2.0;
     if (!(lo == hi)) {
         double spt = 0;
-        for (uint32_t s = threadIdx.x; s < Np; s += kPlainThreads) {
+        for (uint32_t s = threadIdx.x; s < Np; s += blockDim.x) {
             const float wp = P.w[c.p0 + (int)s];
             if (c.pr.caseA) {
                 spt += (double)fminf(wp, I.w[c.t0 + c.pr.pair_of_slot(s) % Nt]);
@@ -714,7 +715,7 @@ __device__ void plain_ei_cell(const CtaGroup& grp, PlainShared& S, const StepArg
     // share the draw of counter q, slot 4q + h its digits 2h and 2h + 1.  A
     // thread per slot (each takes its own copy of the draw), so that small
     // cells keep their threads busy.
-    for (uint32_t s = threadIdx.x; s < c.Np; s += kPlainThreads) {
+    for (uint32_t s = threadIdx.x; s < c.Np; s += blockDim.x) {
         const uint32_t q = s >> 2, h = s & 3u;
         const int sl = c.p0 + (int)s;
         const float ux = P.ux[sl], uy = P.uy[sl], uz = P.uz[sl];
@@ -805,7 +806,7 @@ __device__ void plain_bh_cell(const CtaGroup& grp, PlainShared& S, const StepArg
     bool absorbed_any = false;
     // one 16-bit accept digit per pair (BH): slots 8q .. 8q + 7 share the
     // draw of counter q, slot 8q + h its digit h; a thread per slot
-    for (uint32_t s = threadIdx.x; s < c.Np; s += kPlainThreads) {
+    for (uint32_t s = threadIdx.x; s < c.Np; s += blockDim.x) {
         const uint32_t q = s >> 3, h = s & 7u;
         const int sl = c.p0 + (int)s;
         const float ux = P.ux[sl], uy = P.uy[sl], uz = P.uz[sl];
@@ -2747,6 +2748,19 @@ extern "C" int pcc_set_schedule(pcc_ctx* ctx, int min_blocks_per_sm, int blocks_
     return PCC_OK;
 }
 
+// Threads of a plain block.  A block waits on the latency of its cell's phases, so
+// once there are more cells than blocks of 128 threads fit on the SMs (8 on each),
+// twice as many blocks of 64 do better: 16384 cells of 256 electrons 318 against
+// 531 us, of 20 electrons 244 against 454, log-normal ones 402 against 511; 2432
+// cells 87 against 115, 64 against 90 and 93 against 110.  With fewer cells the SMs
+// have room, and a cell is done sooner by 128 threads (64 cells 33 against 36 us,
+// log-normal ones 35 against 42).  Blocks of one warp take 238 us for the first of
+// these, but a large cell holds them up (log-normal ones 548 us).
+static int plain_threads(const pcc_ctx* ctx, int n_cells)
+{
+    return n_cells > 8 * ctx->num_sms ? kPlainThreads / 2 : kPlainThreads;
+}
+
 int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_species* ep, pcc_species* ph,
                    const pcc_species* ion, double dt, uint64_t seed, uint64_t step, unsigned mask, int precision,
                    float* ledger, cudaStream_t st, int (*after_group)(void* user, int group), void* user,
@@ -2799,9 +2813,10 @@ int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_sp
         if (e != cudaSuccess) return cuda_fail(e, "pcc_collide: launch");
         if (run[g]) {
             if (precision == PCC_FP64_PLAIN) {
-                if (g == kGroupEm) launch_pdl(collide_plain_kernel<kGroupEm>, cells->n_cells, kPlainThreads, 0, st, a);
-                else if (g == kGroupEp) launch_pdl(collide_plain_kernel<kGroupEp>, cells->n_cells, kPlainThreads, 0, st, a);
-                else launch_pdl(collide_plain_kernel<kGroupPh>, cells->n_cells, kPlainThreads, 0, st, a);
+                const int threads = plain_threads(ctx, cells->n_cells);
+                if (g == kGroupEm) launch_pdl(collide_plain_kernel<kGroupEm>, cells->n_cells, threads, 0, st, a);
+                else if (g == kGroupEp) launch_pdl(collide_plain_kernel<kGroupEp>, cells->n_cells, threads, 0, st, a);
+                else launch_pdl(collide_plain_kernel<kGroupPh>, cells->n_cells, threads, 0, st, a);
                 note_launches(1);
             } else {
                 if (g == kGroupEm) e = launch_batched<kGroupEm>(ctx, a, stage, st);
