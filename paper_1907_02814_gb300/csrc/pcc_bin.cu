@@ -81,8 +81,7 @@ __device__ __forceinline__ unsigned near_peers(int c)
 }
 
 // One global atomic per group of lanes.
-__global__ void bin_count_kernel(const int* __restrict__ cell, int n, int n_cells, int* __restrict__ counts,
-                                 DevStats* st)
+__global__ void bin_count_kernel(const int* cell, int n, int n_cells, int* counts, DevStats* st)
 {
     pdl_begin();
     const int c = valid_cell(cell, blockIdx.x * blockDim.x + threadIdx.x, n, n_cells, st);
@@ -94,8 +93,8 @@ __global__ void bin_count_kernel(const int* __restrict__ cell, int n, int n_cell
 // Few cells: a block counts a contiguous chunk of the input in shared memory
 // and adds a cell's count once: 2048 cells of 8192 shuffled particles 0.70 -> 0.06
 // ms (a global atomic per particle before).
-__global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) bin_count_local_kernel(const int* __restrict__ cell, int n, int n_cells,
-                                                                           int* __restrict__ counts, DevStats* st)
+__global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) bin_count_local_kernel(const int* cell, int n, int n_cells,
+                                                                                      int* counts, DevStats* st)
 {
     pdl_begin();
     extern __shared__ int h[];
@@ -124,8 +123,8 @@ struct BlockSums {
     int particles, largest;
 };
 
-__global__ void __launch_bounds__(kScanBlock) region_sums_kernel(const int* __restrict__ counts, int n, int slack_abs,
-                                                                 double slack_rel, BlockSums* __restrict__ sums)
+__global__ void __launch_bounds__(kScanBlock) region_sums_kernel(const int* counts, int n, int slack_abs,
+                                                                 double slack_rel, BlockSums* sums)
 {
     pdl_begin();
     __shared__ long long s[32];
@@ -164,13 +163,10 @@ __device__ __forceinline__ int sort_class(int count)
 // Each block adds up the sums of the blocks before it and scans its own cells:
 // the atomic maximum of every cell alone took 64 us of a 1e5-cell binning, and
 // one thread walked the block sums.
-__global__ void __launch_bounds__(kScanBlock) region_offsets_kernel(const BlockSums* __restrict__ sums, int nb,
-                                                                    const int* __restrict__ counts, int n, int slack_abs,
-                                                                    double slack_rel, int* __restrict__ cell_start,
-                                                                    int* __restrict__ cell_count,
-                                                                    int* __restrict__ cell_added, int* __restrict__ first,
-                                                                    int* __restrict__ cursor, BinTotals* __restrict__ totals,
-                                                                    SortLists L)
+__global__ void __launch_bounds__(kScanBlock) region_offsets_kernel(const BlockSums* sums, int nb, const int* counts, int n,
+                                                                    int slack_abs, double slack_rel, int* cell_start,
+                                                                    int* cell_count, int* cell_added, int* first,
+                                                                    int* cursor, BinTotals* totals, SortLists L)
 {
     pdl_begin();
     __shared__ long long sl[32];
@@ -277,8 +273,7 @@ __device__ __forceinline__ void store_record(const MRec& out, int dst, const Tmp
     out.pid[dst] = (uint64_t)r.pid_hi << 32 | r.pid_lo;
 }
 
-__global__ void bin_scatter_kernel(Rec in, const int* __restrict__ cell, int n, int n_cells, int* __restrict__ cursor,
-                                   TmpRec* __restrict__ tmp, BinLimits lim)
+__global__ void bin_scatter_kernel(Rec in, const int* cell, int n, int n_cells, int* cursor, TmpRec* tmp, BinLimits lim)
 {
     pdl_begin();
     if (lim.exceeded()) return;
@@ -298,9 +293,9 @@ __global__ void bin_scatter_kernel(Rec in, const int* __restrict__ cell, int n, 
 // 4096 particles keep the records that are being filled in (32 B each, all
 // blocks) within L2, so that its lines reach memory whole.
 constexpr int kTileItems = 8;
-__global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) bin_scatter_local_kernel(Rec in, const int* __restrict__ cell, int n,
-                                                                             int n_cells, int* __restrict__ cursor,
-                                                                             TmpRec* __restrict__ tmp, BinLimits lim)
+__global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) bin_scatter_local_kernel(Rec in, const int* cell, int n,
+                                                                                        int n_cells, int* cursor,
+                                                                                        TmpRec* tmp, BinLimits lim)
 {
     pdl_begin();
     extern __shared__ int h[];
@@ -618,11 +613,9 @@ __device__ __forceinline__ void sort_cell_warp(SortSmem<1, ITEMS>& S, const TmpR
 
 // A warp per cell of up to kSortWarpCap records; up to 64 by counting the smaller pids.
 constexpr int kSortWarps = 4;
-__global__ void __launch_bounds__(32 * kSortWarps, 12) sort_warp_kernel(const int* __restrict__ cell_start,
-                                                                        const int* __restrict__ cell_count,
-                                                                        const int* __restrict__ first, int n_cells,
-                                                                        const TmpRec* __restrict__ tmp, MRec out,
-                                                                        BinLimits lim)
+__global__ void __launch_bounds__(32 * kSortWarps, 12) sort_warp_kernel(const int* cell_start, const int* cell_count,
+                                                                        const int* first, int n_cells, const TmpRec* tmp,
+                                                                        MRec out, BinLimits lim)
 {
     pdl_begin();
     constexpr unsigned kFull = 0xffffffffu;
@@ -656,11 +649,9 @@ __global__ void __launch_bounds__(32 * kSortWarps, 12) sort_warp_kernel(const in
 
 // A block per cell of one class's list.
 template <int W, int ITEMS>
-__global__ void __launch_bounds__(32 * W, W == 4 ? 8 : 32 / ITEMS) sort_block_kernel(const int* __restrict__ cell_start,
-                                                            const int* __restrict__ cell_count,
-                                                            const int* __restrict__ first, const int* __restrict__ list,
-                                                            const int* __restrict__ count, const TmpRec* __restrict__ tmp,
-                                                            MRec out, BinLimits lim)
+__global__ void __launch_bounds__(32 * W, W == 4 ? 8 : 32 / ITEMS) sort_block_kernel(const int* cell_start, const int* cell_count,
+                                                            const int* first, const int* list, const int* count,
+                                                            const TmpRec* tmp, MRec out, BinLimits lim)
 {
     pdl_begin();
     extern __shared__ __align__(16) unsigned char sort_smem[];
@@ -684,7 +675,7 @@ __global__ void commit_kernel(SpeciesView sp, int n_cells)
 
 // ---- FP64 totals: slots shared out to the warps, fixed-order partials per block (see pcc_totals.cuh)
 template <bool PHOTON>
-__global__ void __launch_bounds__(256, 4) totals_kernel(const pcc_species sp, int n_cells, double* __restrict__ partial)
+__global__ void __launch_bounds__(256, 4) totals_kernel(const pcc_species sp, int n_cells, double* partial)
 {
     pdl_begin();
     __shared__ double sh[3][32];

@@ -22,7 +22,10 @@ constexpr double kPi = 3.14159265358979323846;
 // First statement of a kernel launched by launch_pdl, on every thread: lets the
 // kernel after it come in as blocks leave, then waits for the one before it to
 // complete, its writes included.  Since every kernel of a chain waits, all
-// earlier ones are complete too.
+// earlier ones are complete too.  Such a kernel is resident while the one before
+// it still writes, so its pointers carry no __restrict__: that would let the
+// compiler take their loads for loads of constant memory and move them over the
+// wait.
 __device__ __forceinline__ void pdl_begin()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
