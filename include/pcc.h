@@ -103,7 +103,11 @@ typedef struct {
  * Cell c owns slots [cell_start[c], cell_start[c+1]); its live particles
  * are the first cell_count[c] slots, in ascending pid order.  Secondaries
  * created during a step are appended after them (cell_added[c]) and become
- * live at pcc_append_secondaries.  x may be NULL.  capacity = total slots. */
+ * live at pcc_append_secondaries.  The slots behind both are free: they hold
+ * what was there before, or copies of records that moved down when absorbed
+ * photons were removed.  The same calls on the same state leave the same bytes
+ * in every slot, unless a region overflows (PCC_ST_CAPACITY).
+ * x may be NULL.  capacity = total slots. */
 typedef struct {
     float *ux, *uy, *uz, *w;
     float *x;

@@ -835,9 +835,9 @@ __device__ void plain_bh_cell(const CtaGroup& grp, PlainShared& S, const StepArg
                 *L = make_float4(v.x, v.y, k2.s, k2.c);
             }
         }
-        if (threadIdx.x == 0) {   // stable compaction of the region (rare path)
+        if (threadIdx.x == 0) {   // stable compaction of the region (rare path), see compact_region_warp
             const bool has_x = P.x != nullptr;
-            const int Np = (int)c.Np, p0 = c.p0, n_all = Np + P.added[cell];
+            const int Np = (int)c.Np, p0 = c.p0, n_all = Np + order_added(P, cell);
             int wr = 0, removed = 0;
             for (int i = 0; i < n_all; ++i) {
                 const int src = p0 + i;
@@ -1906,9 +1906,11 @@ __global__ void __launch_bounds__(kBatchedThreads, 2) caseb_cand_kernel(const __
 
 // Stable removal of the absorbed photons (weight 0) from the first Np slots
 // of a cell region, keeping the order of the rest (including the Np..n_all
-// secondaries appended in this step), one warp.  The records before the
-// first removed one are not touched; from there each batch of 4 x 32
-// records is read into registers before any of it is written, and
+// secondaries appended in this step), one warp.  The secondaries are put in
+// pid order first: the slots that the move vacates keep copies of the last of
+// them, which would otherwise be those that happened to arrive last.  The
+// records before the first removed one are not touched; from there each batch
+// of 4 x 32 records is read into registers before any of it is written, and
 // destinations never pass sources.
 __device__ void compact_region_warp(const SpeciesView& P, int cell)
 {
@@ -1931,6 +1933,8 @@ __device__ void compact_region_warp(const SpeciesView& P, int cell)
         if (__any_sync(kFull, hole)) break;
     }
     if (c0 >= Np) return;   // nothing removed
+    if (lane == 0) order_added(P, cell);
+    __syncwarp();
     int wr = c0;            // warp-uniform write position
     for (int b = c0; b < n_all; b += 32 * kU) {
         float ux[kU], uy[kU], uz[kU], w[kU], x[kU];

@@ -18,11 +18,12 @@ __host__ __device__ inline SpeciesView view_of(const pcc_species& s)
     return SpeciesView{s.ux, s.uy, s.uz, s.w, s.x, s.pid, s.cell_start, s.cell_count, s.cell_added};
 }
 
-// Orders the records appended to cell c by pid and makes them live.
-__device__ __forceinline__ void commit_cell(const SpeciesView& sp, int c)
+// Orders the records appended to cell c by pid (they arrive in the order of
+// atomics) and returns their number.
+__device__ __forceinline__ int order_added(const SpeciesView& sp, int c)
 {
     const int a = sp.added[c];
-    if (a == 0) return;
+    if (a == 0) return 0;
     const int b = sp.start[c] + sp.count[c];
     for (int i = 1; i < a; ++i) {   // insertion sort of the (few) appended records
         const uint64_t kp = sp.pid[b + i];
@@ -42,6 +43,14 @@ __device__ __forceinline__ void commit_cell(const SpeciesView& sp, int c)
         sp.ux[b + j + 1] = vx; sp.uy[b + j + 1] = vy; sp.uz[b + j + 1] = vz; sp.w[b + j + 1] = vw;
         if (sp.x) sp.x[b + j + 1] = vxx;
     }
+    return a;
+}
+
+// Orders the records appended to cell c and makes them live.
+__device__ __forceinline__ void commit_cell(const SpeciesView& sp, int c)
+{
+    const int a = order_added(sp, c);
+    if (a == 0) return;
     sp.count[c] += a;
     sp.added[c] = 0;
 }
