@@ -35,7 +35,7 @@
 // relativistic nodes (gamma <= 2) use q_+^2 - q_-^2 = 4 p1 p2, so that the
 // logarithms of the Yukawa terms are those of the cross term, or FP64 in cells
 // where L_D is within 5 % of L_TF, where the cross term's divided difference
-// cancels.  Sums over a lane's nodes and samples are compensated FP32, over
+// cancels (or where a length is beyond 1e15).  Sums over a lane's nodes and samples are compensated FP32, over
 // lanes and warps FP64.
 //
 // Adjoint.  The parameters enter only through the screening quantities
@@ -203,6 +203,8 @@ struct RelCell {
     float L, iL, i1L2, rho, rhop, ln1L2, ln1L2_lo, l1pi;
 };
 
+constexpr double kNrMax = 1e30;   // largest L^2 of the FP32 non-relativistic nodes (12 L^2 is a normal float)
+
 struct CellScreen {
     double LTF, LD, etaTF, etaD, a, LR;
     double n_i, T_e, Zs, sTF, sD;
@@ -210,7 +212,7 @@ struct CellScreen {
     // derivatives of L_R through a = I_TFD (adjoint only)
     double LR_eD, LR_LTF, LR_LD;
     bool debye;   // lambda_D > r_i (the Debye branch of L_D is active)
-    bool nr32;    // L_D and L_TF far enough apart for the FP32 non-relativistic branch
+    bool nr32;    // L_D and L_TF far enough apart, and small enough, for the FP32 non-relativistic branch
     bool ok;
 };
 
@@ -242,7 +244,7 @@ __device__ CellScreen cell_screen(const float* p, int Z)
     const double w = lambert_w0_neg(-exp(-1.0 - 2.0 * c.a));
     c.LR = sqrt(expm1(w + 1.0 + 2.0 * c.a));
     const double A = c.LTF * c.LTF, B = c.LD * c.LD;
-    c.nr32 = fabs(B - A) > 0.05 * fmax(A, B);
+    c.nr32 = fabs(B - A) > 0.05 * fmax(A, B) && fmax(A, B) < kNrMax;
     const double x = c.LR * c.LR, ix = 1.0 / (1.0 + x);
     const double ln = log1p(x);
     c.rel = RelCell{(float)c.LR, (float)(1.0 / c.LR), (float)ix, (float)(x * ix), (float)(2.0 * c.LR * ix * ix),
@@ -436,6 +438,7 @@ __device__ __forceinline__ void rel_nodes(const EmArgs& a, const RelCell& L, flo
 // What the non-relativistic nodes need of the screening.
 struct NrCell {
     float A, B, iBA, eT, eD, LTF2, LD2;   // L_TF^2, L_D^2, 1/(B - A), eta_TF, eta_D, 2 L_TF, 2 L_D
+    float kA, kB;                         // B/(B - A) 2 L_TF, A/(B - A) 2 L_D
 };
 
 // Nodes [q0, q1) of one sample with gamma <= 2 (per lane), Eq. (cs_br_nr) with the
@@ -443,8 +446,11 @@ struct NrCell {
 // P = q+^2 - q-^2 = 4 p1 p2 exactly, T-+ = 1 + q-+^2 A, D-+ = 1 + q-+^2 B,
 // la = ln(T+/T-) = log1p(P A / T-), lb likewise, the bracket is
 //   eta_TF^2/2 (la - P A/(T+ T-)) + eta_D^2/2 (lb - P B/(D+ D-)) + eta_TF eta_D X,
-//   X = (B la - A lb)/(B - A):
-// no difference of nearly equal numbers is formed.
+//   X = (B la - A lb)/(B - A),
+//   dX/dA = B (P/(T+ T-) - (lb - la)/(B - A))/(B - A), dX/dB = A ((lb - la)/(B - A) - P/(D+ D-))/(B - A):
+// no difference of nearly equal numbers is formed.  Every factor has a reciprocal
+// of its own: B reaches 1e22 in thin plasmas (and kNrMax), and the product D+ D-
+// passes the FP32 range from L_D = 1e9 on.
 template <bool GRAD>
 __device__ __forceinline__ void nr_nodes(const EmArgs& a, const NrCell& C, float g, float bw, int q0, int q1, Acc& acc)
 {
@@ -463,19 +469,20 @@ __device__ __forceinline__ void nr_nodes(const EmArgs& a, const NrCell& C, float
         const float ib2 = (1.0f + T2) * rcp_nr(p2);
         const float pre = pre1 * ib2 * rcp_nr(-expm1f(-az * ib2));
         const float Tm = fmaf(qm2, C.A, 1.0f), Tp = fmaf(qp2, C.A, 1.0f), Dm = fmaf(qm2, C.B, 1.0f), Dp = fmaf(qp2, C.B, 1.0f);
-        const float it = rcp_nr(Tm * Tp), id = rcp_nr(Dm * Dp), PA = P * C.A, PB = P * C.B;
-        const float la = log1pf(PA * Tp * it), lb = log1pf(PB * Dp * id);
-        const float gT = la - PA * it, gD = lb - PB * id, X = (C.B * la - C.A * lb) * C.iBA;
+        const float iTm = rcp_nr(Tm), iTp = rcp_nr(Tp), iDm = rcp_nr(Dm), iDp = rcp_nr(Dp);
+        const float ya = P * C.A * iTm, yb = P * C.B * iDm;   // T+/T- - 1, D+/D- - 1
+        const float la = log1pf(ya), lb = log1pf(yb);
+        const float gT = la - ya * iTp, gD = lb - yb * iDp, X = (C.B * la - C.A * lb) * C.iBA;
         float f = pre * (0.5f * C.eT * C.eT * gT + 0.5f * C.eD * C.eD * gD + C.eT * C.eD * X);
         float df[3];
         if (GRAD) {
-            const float dX_A = (PB * it - lb + X) * C.iBA, dX_B = (la - PA * id - X) * C.iBA;
-            const float dgT = PA * it * it * (qm2 * Tp + qp2 * Tm), dgD = PB * id * id * (qm2 * Dp + qp2 * Dm);
-            df[0] = pre * (0.5f * C.eT * C.eT * dgT + C.eT * C.eD * dX_A) * C.LTF2;
-            df[1] = pre * (0.5f * C.eD * C.eD * dgD + C.eT * C.eD * dX_B) * C.LD2;
+            const float dl = (lb - la) * C.iBA;
+            const float dgT = C.LTF2 * iTp * ya * (qm2 * iTm + qp2 * iTp), dgD = C.LD2 * iDp * yb * (qm2 * iDm + qp2 * iDp);
+            df[0] = pre * (0.5f * C.eT * C.eT * dgT + C.eT * C.eD * (C.kA * (P * iTm * iTp - dl)));
+            df[1] = pre * (0.5f * C.eD * C.eD * dgD + C.eT * C.eD * (C.kB * (dl - P * iDm * iDp)));
             df[2] = pre * (-C.eT * gT + C.eD * gD + (C.eT - C.eD) * X);
         }
-        if (!(f > 0.f)) {
+        if (f <= 0.f) {
             f = 0.f;
             if (GRAD) df[0] = df[1] = df[2] = 0.f;
         }
@@ -638,6 +645,9 @@ __global__ void __launch_bounds__(kEmThreads, GRAD ? 3 : 4) emission_kernel(cons
             C.eD = (float)cs.etaD;
             C.LTF2 = 2.0f * (float)cs.LTF;
             C.LD2 = 2.0f * (float)cs.LD;
+            const double A = cs.LTF * cs.LTF, B = cs.LD * cs.LD;
+            C.kA = (float)(2.0 * cs.LTF * B / (B - A));
+            C.kB = (float)(2.0 * cs.LD * A / (B - A));
             deal_nodes(n_nr, a.n_quad, [&](int i, int q0, int q1) {
                 nr_nodes<GRAD>(a, C, list[1][i].x, list[1][i].y, q0, q1, acc);
             });
