@@ -311,6 +311,7 @@ __device__ __forceinline__ Panel panel_of(int p, int nc, bool logcol, double ly)
 // 31 materials x 256 x 256, 8 nodes: Brems 28.7 -> 4.1 ms, Bethe-Heitler 34.2 -> 2.2 ms;
 // one material in the full potential: 24.3 -> 1.5 and 11.8 -> 0.8 ms.
 constexpr int kBlockMats = 8, kRowThreads = 256;
+constexpr int kRowSmem = 96 * 1024;   // dynamic shared memory of a block at most
 
 template <int KIND>
 __global__ void __launch_bounds__(kRowThreads) table_rows_kernel(const double* screen, const double* tfd, int n_mats,
@@ -516,15 +517,17 @@ extern "C" int pcc_tables_build(pcc_ctx* ctx, const pcc_material* mats, int n_ma
     legendre_nodes(kTfdNodes, rule.tx, rule.tw);
     int group = 1;                          // lanes per panel: a power of two, at least the nodes
     while (group < s.quad_nodes) group <<= 1;
-    // materials per block: their columns in at most 96 KB of shared memory
     const size_t row_bytes = (C + 2 * (kEdgePanels + 1)) * sizeof(double);
-    const int per = std::max(1, std::min({kBlockMats, n_mats, (int)(96 * 1024 / row_bytes)}));
+    const int per = std::max(1, std::min({kBlockMats, n_mats, (int)(kRowSmem / row_bytes)}));
     const int chunks = (n_mats + per - 1) / per, per_block = (n_mats + chunks - 1) / chunks;
     const size_t smem = per_block * row_bytes;
-    if (smem > 48 * 1024) {
-        cudaFuncSetAttribute(table_rows_kernel<kBrems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(table_rows_kernel<kBH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    }
+    // Always the same limit: without it a block's static and dynamic shared memory
+    // together may not pass 48 KB, and a limit set per call would be another
+    // thread's too.
+    e = cudaFuncSetAttribute(table_rows_kernel<kBrems>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(table_rows_kernel<kBH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem);
+    if (e != cudaSuccess) { free_tables(ctx); cudaFree(dmats); return cuda_fail(e, "pcc_tables_build: shared memory"); }
     double* tfd = nullptr;
     if (flags & kFlagTfdQuad) {
         e = cudaMalloc(&tfd, M * (kTfdPanels + 1) * kTfdMoments * sizeof(double));
