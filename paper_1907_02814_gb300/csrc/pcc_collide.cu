@@ -1509,9 +1509,10 @@ __device__ __forceinline__ void scan_segment(const StepArgs& a, const CellList& 
             const float bm = fminf(bmax, 1.f);
             bfac = fminf((1.f + (bm > 0.f ? bm * rsqrtf(bm) : 0.f)) * (1.f + 0x1p-20f), 2.f);
         }
-        if constexpr (kWriter) {
+        if constexpr (kWriter) {   // uniform only if every lane of the group saw equal weights
+            const unsigned odd = __ballot_sync(kFull, !uni);
             if (active && gl == 0)
-                IC.sum[cell] = make_float4(n_t, w0, uni ? bfac : -bfac, __uint_as_float(*IC.serial));
+                IC.sum[cell] = make_float4(n_t, w0, odd & gmask ? -bfac : bfac, __uint_as_float(*IC.serial));
         }
         if (caseA) {
             // the weights as float4 from the region's first 16-byte boundary
