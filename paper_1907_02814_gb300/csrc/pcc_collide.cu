@@ -718,8 +718,11 @@ __device__ void plain_ei_cell(const CtaGroup& grp, PlainShared& S, const StepArg
     for (uint32_t s = threadIdx.x; s < c.Np; s += blockDim.x) {
         const uint32_t q = s >> 2, h = s & 3u;
         const int sl = c.p0 + (int)s;
-        const float ux = P.ux[sl], uy = P.uy[sl], uz = P.uz[sl];
-        const bool below = plainly_below(1.f + (ux * ux + uy * uy + uz * uz), c.reach2, limit);
+        const auto is_below = [&] {
+            const float ux = P.ux[sl], uy = P.uy[sl], uz = P.uz[sl];
+            return plainly_below(1.f + (ux * ux + uy * uy + uz * uz), c.reach2, limit);
+        };
+        bool below = is_below();
         const uint32_t passes = c.pr.caseA ? 1u : (c.Nt - s + c.Np - 1) / c.Np;
         for (uint32_t m = 0; m < passes; ++m) {
             const Philox4 ac = draw_k(q, cell, (uint32_t)a.step, stream_tag(group, kAccept, m), a.keys);
@@ -727,7 +730,10 @@ __device__ void plain_ei_cell(const CtaGroup& grp, PlainShared& S, const StepArg
             if (below && rB > kB && rT > kT) continue;
             const uint32_t j = c.pr.caseA ? c.pr.pair_of_slot(s) : s + m * c.Np;
             const uint32_t t = c.pr.caseA ? j % c.Nt : c.pr.target_of_pair(j);
-            had |= plain_ei_pair(&a, group, &c, s, j, t, rB, rT, m, &S.acc, &ev);
+            if (plain_ei_pair(&a, group, &c, s, j, t, rB, rT, m, &S.acc, &ev)) {
+                had = true;
+                below = is_below();   // losing energy to a moving ion can raise it in the simulation frame
+            }
         }
         // the full path counts every pair of such a cell as a candidate
         if (!c.pr.caseA) atomicAdd(&S.acc.candidates[group], (unsigned long long)passes);
