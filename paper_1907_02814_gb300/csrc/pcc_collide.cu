@@ -902,8 +902,10 @@ struct CellList {
 // against 103-118 us, log-normal ones 65-89 against 120-136 us; at 32768 cells
 // 84-152 against 109-148 us and for log-normal ones 122-179 against 131-165 us,
 // since the large cells, which the general scan takes first, hold up a warp.
-// (Log-normal cells with as many ions as electrons in a step so long that large
-// cells collide on most pairs are the exception: 490 against 280 us at 16384.)
+// Steps so long that large cells collide on most pairs take the longest on one
+// warp, so its block works off long candidate lists together (see
+// fused_lists_block): 16384 log-normal cells with as many ions as electrons at
+// 1 fs 445 -> 265 us, the general sequence 277.
 constexpr int kFusedMinCells = 32;
 constexpr int kFusedCellsPerWarp = 5;
 constexpr int kFusedWarpsPerSM = 24;
@@ -1803,18 +1805,41 @@ __device__ __forceinline__ bool flat_pair(const StepArgs& a, const Tab<float>& t
     return eval_pair<PH>(a, tb, group, cell, cm, s, j, fast_mod(j, cm.Nt, 1.0f / (float)cm.Nt), 0u, acc, rad, wcre);
 }
 
+// Up to 32 candidates of a cell with N_p < N_t, a lane each (pair j where valid):
+// candidates of the same projectile among them one after the other, since its
+// momentum after one event enters the next and an absorbed photon skips its later
+// pairs.  tab: the P table of lists of at most 32 targets.  True when the lane
+// changed a projectile.
+template <bool PH>
+__device__ __forceinline__ bool caseb_chunk(const StepArgs& a, const Tab<float>& tb, int group, int cell, const CellRec& cm,
+                                            bool valid, uint32_t j, const int* tab, const PermKeys& rk, int lane, Acc& acc,
+                                            float& rad, float& wcre)
+{
+    const uint32_t Np = cm.Np, Nt = cm.Nt, m = j / Np, s = j - m * Np;
+    const unsigned peers = __match_any_sync(0xffffffffu, valid ? s : 0x80000000u | (uint32_t)lane);
+    const int turn = __popc(peers & ((1u << lane) - 1u));
+    const int turns = __reduce_max_sync(0xffffffffu, turn);
+    bool any = false;
+    for (int r = 0; r <= turns; ++r) {
+        if (valid && turn == r && !(PH && a.ph.w[cm.p0 + (int)s] == 0.f)) {
+            const uint32_t t = Nt <= 32 ? (uint32_t)tab[j] : perm_elem_large(j, Nt, rk);
+            any |= eval_pair<PH>(a, tb, group, cell, cm, s, j, t, m, acc, rad, wcre);
+        }
+        __syncwarp();
+    }
+    return any;
+}
+
 // The cnt candidates (pair indices qb, increasing for each projectile) of a
-// cell with N_p < N_t, by all 32 lanes: a lane per candidate, and candidates of
-// the same projectile among them one after the other, since its momentum after
-// one event enters the next and an absorbed photon skips its later pairs.  (On
-// one lane the list of a large cell was the longest chain of the call.)  tab:
-// 32 ints for the P table of short lists.  True when the lane changed a projectile.
+// cell with N_p < N_t, by all 32 lanes (see caseb_chunk; on one lane the list
+// of a large cell was the longest chain of the call).  tab: 32 ints for the P
+// table of short lists.  True when the lane changed a projectile.
 template <bool PH>
 __device__ __forceinline__ bool caseb_pairs(const StepArgs& a, const Tab<float>& tb, int group, int cell, const CellRec& cm,
                                             const uint32_t* qb, int cnt, int* tab, int lane, Acc& acc, float& rad,
                                             float& wcre)
 {
-    const uint32_t Np = cm.Np, Nt = cm.Nt;
+    const uint32_t Nt = cm.Nt;
     const PermKeys rk = perm_keys(a, group, cell);
     __syncwarp();
     if (Nt <= 32 && lane < (int)Nt) tab[perm_pos_small(lane, Nt, rk)] = lane;   // P table of the targets
@@ -1822,18 +1847,7 @@ __device__ __forceinline__ bool caseb_pairs(const StepArgs& a, const Tab<float>&
     bool any = false;
     for (int k0 = 0; k0 < cnt; k0 += 32) {
         const bool valid = k0 + lane < cnt;
-        const uint32_t j = valid ? qb[k0 + lane] : 0u;
-        const uint32_t m = j / Np, s = j - m * Np;
-        const unsigned peers = __match_any_sync(0xffffffffu, valid ? s : 0x80000000u | (uint32_t)lane);
-        const int turn = __popc(peers & ((1u << lane) - 1u));
-        const int turns = __reduce_max_sync(0xffffffffu, turn);
-        for (int r = 0; r <= turns; ++r) {
-            if (valid && turn == r && !(PH && a.ph.w[cm.p0 + (int)s] == 0.f)) {
-                const uint32_t t = Nt <= 32 ? (uint32_t)tab[j] : perm_elem_large(j, Nt, rk);
-                any |= eval_pair<PH>(a, tb, group, cell, cm, s, j, t, m, acc, rad, wcre);
-            }
-            __syncwarp();
-        }
+        any |= caseb_chunk<PH>(a, tb, group, cell, cm, valid, valid ? qb[k0 + lane] : 0u, tab, rk, lane, acc, rad, wcre);
     }
     return any;
 }
@@ -2038,18 +2052,25 @@ __global__ void finalize_kernel(const __grid_constant__ StepArgs a, Queue Q)
 struct FusedArgs {
     int thr[3][4];      // scan lane groups per group (see CellList)
     unsigned run;       // bit g: group g takes part
-    uint32_t* qb;       // [target capacity] pair indices of candidates in cells with N_p < N_t
+    // Per group, candidates that do not wait in shared memory, at their cell's own
+    // place: slots [projectile capacity] of cells with N_p >= N_t, pair indices
+    // [target capacity] of the others.
+    uint32_t *flat[3], *qb[3];
+    uint32_t cap[3];    // projectile capacities
 };
 
 constexpr int kFusedWarps = kBatchedThreads / 32;
 constexpr int kFusedBatch = 8;      // cells scanned before their candidates are evaluated
 constexpr int kFusedQueue = 1024;   // staged candidates: all that one pass of the accept loop can mark
+constexpr int kFusedOwn = 64;       // candidates with N_p < N_t up to which a cell's warp takes them itself
+constexpr uint32_t kFusedSlots = 1u << 27;   // staged slots are below this
 
 struct FusedWarp {
     float2 ev[kFusedBatch][3];      // radiated energy and created weight of the cell's events
-    struct { int p0; uint32_t Np; float coef; int cnt_b; } rec[kFusedBatch][3];   // cnt_b: candidates if N_p < N_t
+    struct { int p0; uint32_t Np; float coef; int cnt; } rec[kFusedBatch][3];   // cnt: entries of its list in FusedArgs
     struct { int cell, t0, mat; uint32_t Nt; } cell[kFusedBatch];
     unsigned changed;               // bit 4b + g: an event in group g of cell b
+    unsigned lists;                 // bit 4b + g: the block works off group g's list of cell b
     int tab[64];
     uint32_t q[kFusedQueue];        // slot << 5 | b << 2 | g
 };
@@ -2081,21 +2102,10 @@ __device__ __forceinline__ void fused_candidate(const StepArgs& a, FusedWarp& w,
     if (event) fused_event(w, b, g, rad, wcre);
 }
 
-// The staged candidates of one warp (when its list is full), or of all warps
-// of the block together, so that a cell full of candidates does not hold
-// up one warp.  Out of line, as the other rare paths, so that the scan of the
-// mostly candidate-free cells keeps its registers (inlined, the kernel spilled
-// 734 bytes).
-__device__ __noinline__ void fused_drain(const StepArgs* ap, FusedWarp* w, int nq, BlockAcc* bacc)
-{
-    __syncwarp();
-    Acc acc;
-    acc.zero();
-    for (int i = threadIdx.x & 31; i < nq; i += 32) fused_candidate(*ap, *w, w->q[i], acc);
-    add_rare(acc, *bacc);
-    __syncwarp();
-}
-
+// The staged candidates of all warps of the block together, so that a cell full
+// of candidates does not hold up one warp.  Out of line, as the other rare paths,
+// so that the scan of the mostly candidate-free cells keeps its registers
+// (inlined, the kernel spilled 734 bytes).
 __device__ __noinline__ void fused_drain_block(const StepArgs* ap, FusedWarp* work, const int* staged, BlockAcc* bacc)
 {
     int total = 0;
@@ -2113,11 +2123,12 @@ __device__ __noinline__ void fused_drain_block(const StepArgs* ap, FusedWarp* wo
 }
 
 // The queued candidates of cell b's group g with N_p < N_t.  All 32 lanes.
-__device__ __noinline__ void fused_caseb(const StepArgs* ap, const uint32_t* qb, FusedWarp* w, int b, int g, BlockAcc* bacc)
+__device__ __noinline__ void fused_caseb(const StepArgs* ap, const uint32_t* qb, FusedWarp* w, int b, int g, int cnt,
+                                         BlockAcc* bacc)
 {
     const StepArgs& a = *ap;
     const Tab<float> tb{a.f_brems_lnsig, a.f_brems_cdf, a.f_bh_lnsig, a.f_bh_cdf, a.f_tri_gp, a.f_tri_split};
-    const int lane = threadIdx.x & 31, cell = w->cell[b].cell, cnt = w->rec[b][g].cnt_b;
+    const int lane = threadIdx.x & 31, cell = w->cell[b].cell;
     const CellRec cm = fused_rec(*w, b, g);
     Acc acc;
     acc.zero();
@@ -2127,6 +2138,78 @@ __device__ __noinline__ void fused_caseb(const StepArgs* ap, const uint32_t* qb,
     if (event) fused_event(*w, b, g, rad, wcre);
     add_rare(acc, *bacc);
     __syncwarp();
+}
+
+// The warp's share of a long list of a cell with N_p < N_t: the candidates of the
+// projectiles whose slot has its number modulo the warps, so that all pairs of a
+// projectile stay with one warp, in order.  The list is read by every warp; those
+// that are its own gather in buf (64 entries) and are evaluated 32 at a time.
+template <bool PH>
+__device__ __forceinline__ bool caseb_share(const StepArgs& a, const Tab<float>& tb, int group, int cell, const CellRec& cm,
+                                            const uint32_t* qb, int cnt, int* buf, int wid, int lane, Acc& acc, float& rad,
+                                            float& wcre)
+{
+    constexpr unsigned kFull = 0xffffffffu;
+    const PermKeys rk = perm_keys(a, group, cell);
+    const unsigned below = (1u << lane) - 1u;
+    bool any = false;
+    int n = 0;   // gathered
+    uint32_t j[4] = {0u, 0u, 0u, 0u};            // four rows of the list are loaded at a time
+    for (int k0 = 0, u = 0; k0 < cnt || n; k0 += 32, u = (u + 1) & 3) {   // warp-uniform
+        if (u == 0)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) j[q] = k0 + 32 * q + lane < cnt ? qb[k0 + 32 * q + lane] : 0u;
+        const uint32_t ju = u == 0 ? j[0] : u == 1 ? j[1] : u == 2 ? j[2] : j[3];
+        const bool own = k0 + lane < cnt && (int)(ju % cm.Np % kFusedWarps) == wid;
+        const unsigned m = __ballot_sync(kFull, own);
+        if (own) buf[n + __popc(m & below)] = (int)ju;
+        n += __popc(m);
+        __syncwarp();
+        if (n >= 32 || k0 + 32 >= cnt) {
+            any |= caseb_chunk<PH>(a, tb, group, cell, cm, lane < n, lane < n ? (uint32_t)buf[lane] : 0u, nullptr, rk, lane, acc,
+                                   rad, wcre);
+            n = max(n - 32, 0);
+            const int rest = buf[32 + lane];
+            __syncwarp();
+            if (lane < n) buf[lane] = rest;
+            __syncwarp();
+        }
+    }
+    return any;
+}
+
+// The long lists of all warps' cells, by the whole block: one warp alone took
+// about 5 us for every 32 candidates of a cell.
+__device__ __noinline__ void fused_lists_block(const StepArgs* ap, const FusedArgs* F, FusedWarp* work, BlockAcc* bacc)
+{
+    const StepArgs& a = *ap;
+    const Tab<float> tb{a.f_brems_lnsig, a.f_brems_cdf, a.f_bh_lnsig, a.f_bh_cdf, a.f_tri_gp, a.f_tri_split};
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    Acc acc;
+    acc.zero();
+    bool some = false;
+    for (int k = 0; k < kFusedWarps; ++k) {
+        FusedWarp& w = work[k];
+        for (unsigned ls = w.lists; ls; ls &= ls - 1u) {   // block-uniform
+            const int bit = __ffs(ls) - 1, b = bit >> 2, g = bit & 3, cnt = w.rec[b][g].cnt, cell = w.cell[b].cell;
+            const CellRec cm = fused_rec(w, b, g);
+            float rad = 0.f, wcre = 0.f;
+            bool event = false;
+            if (cm.Np >= cm.Nt) {
+                const uint32_t* list = F->flat[g] + cm.p0;
+                for (int i = threadIdx.x; i < cnt; i += kBatchedThreads)
+                    event |= g == kGroupPh ? flat_pair<true>(a, tb, g, cell, cm, list[i], acc, rad, wcre)
+                                           : flat_pair<false>(a, tb, g, cell, cm, list[i], acc, rad, wcre);
+            } else {
+                const uint32_t* list = F->qb[g] + cm.t0;
+                event = g == kGroupPh ? caseb_share<true>(a, tb, g, cell, cm, list, cnt, work[wid].tab, wid, lane, acc, rad, wcre)
+                                      : caseb_share<false>(a, tb, g, cell, cm, list, cnt, work[wid].tab, wid, lane, acc, rad, wcre);
+            }
+            if (event) fused_event(w, b, g, rad, wcre);
+            some = true;
+        }
+    }
+    if (some) add_rare(acc, *bacc);
 }
 
 // Cell b's ledger (the groups in order) and the removal of its absorbed photons.
@@ -2182,7 +2265,8 @@ struct IonSums {
 };
 
 // Scan of one group of cell b of the batch: sums, coefficient, accept digits;
-// candidates staged in w.q (nq of them so far) or, with N_p < N_t, in F.qb.
+// candidates staged in w.q (nq of them so far) while there is room, else listed
+// at the cell's place in F; with N_p < N_t always there.
 template <int GROUP>
 __device__ __forceinline__ void fused_scan(const StepArgs& a, const FusedArgs& F, FusedWarp& w, int b, int cell, int p0,
                                            uint32_t Np, int t0, uint32_t Nt, int mat, IonSums& is, int& nq, int lane,
@@ -2270,6 +2354,7 @@ __device__ __forceinline__ void fused_scan(const StepArgs& a, const FusedArgs& F
         constexpr uint32_t kIt = 32 / S;   // iterations per candidate mask
         const uint32_t nit = (Np + S * 32 - 1) / (S * 32);
         const PhiloxFixed pf = philox_fixed((uint32_t)cell, step32, stream_tag(GROUP, kAccept, 0), a.keys);
+        int listed = 0;
 #pragma unroll 1
         for (uint32_t it0 = 0; it0 < nit; it0 += kIt) {
             const uint32_t ite = min(it0 + kIt, nit);
@@ -2292,20 +2377,29 @@ __device__ __forceinline__ void fused_scan(const StepArgs& a, const FusedArgs& F
             }
             const int total = (int)__shfl_sync(kFull, incl, 31);
             if (lane == 0) atomicAdd(&bacc.candidates[GROUP], (unsigned long long)total);
-            if (nq + total > kFusedQueue) {
-                fused_drain(&a, &w, nq, &bacc);
-                nq = 0;
+            const bool stage = nq + total <= kFusedQueue && Np <= kFusedSlots;
+            if (!stage && (uint32_t)p0 + Np > F.cap[GROUP]) {   // a region past the capacity that the caller gave
+                if (lane == 0) atomicOr(&bacc.status, PCC_ST_CAPACITY);
+                continue;
             }
-            uint32_t k = (uint32_t)nq + incl - n;
+            uint32_t* out = stage ? w.q + nq : F.flat[GROUP] + p0 + listed;
+            uint32_t k = incl - n;
 #pragma unroll 1
             while (cmask) {
                 const uint32_t c = (uint32_t)(__ffs(cmask) - 1);
                 cmask &= cmask - 1u;
-                w.q[k++] = (((it0 + c / S) * 32 + (uint32_t)lane) * S + c % S) << 5 | (uint32_t)b << 2 | (uint32_t)GROUP;
+                const uint32_t s = ((it0 + c / S) * 32 + (uint32_t)lane) * S + c % S;
+                out[k++] = stage ? s << 5 | (uint32_t)b << 2 | (uint32_t)GROUP : s;
             }
-            nq += total;
+            if (stage) nq += total;
+            else listed += total;
+        }
+        if (listed && lane == 0) {
+            w.rec[b][GROUP].cnt = listed;
+            w.lists |= 1u << (4 * b + GROUP);
         }
     } else {
+        uint32_t* qb = F.qb[GROUP] + t0;
         const unsigned below = (1u << lane) - 1u;
         const uint32_t Qn = (Np + S - 1) / S, units = Qn * ((Nt + Np - 1) / Np);
         const float inv_qn = 1.0f / (float)Qn;
@@ -2328,18 +2422,20 @@ __device__ __forceinline__ void fused_scan(const StepArgs& a, const FusedArgs& F
 #pragma unroll
             for (int h = 0; h < (int)S; ++h) {
                 const unsigned m = __ballot_sync(kFull, c[h]);
-                if (c[h]) F.qb[t0 + cnt + __popc(m & below)] = S * q + h + mp * Np;
+                if (c[h]) qb[cnt + __popc(m & below)] = S * q + h + mp * Np;
                 cnt += __popc(m);
             }
         }
         if (cnt) {   // warp-uniform
-            // the three groups share the cell's part of qb, so its list is worked off now
             if (lane == 0) {
                 atomicAdd(&bacc.candidates[GROUP], (unsigned long long)cnt);
-                w.rec[b][GROUP].cnt_b = (int)cnt;
+                if (cnt > kFusedOwn) {
+                    w.rec[b][GROUP].cnt = (int)cnt;
+                    w.lists |= 1u << (4 * b + GROUP);
+                }
             }
             __syncwarp();
-            fused_caseb(&a, F.qb, &w, b, GROUP, &bacc);
+            if (cnt <= kFusedOwn) fused_caseb(&a, F.qb[GROUP], &w, b, GROUP, (int)cnt, &bacc);
         }
     }
 }
@@ -2361,7 +2457,7 @@ __global__ void __launch_bounds__(kBatchedThreads, 3) fused_cell_kernel(const __
         const int first = cell;
         int nq = 0, nb = 0;
         if (lane < 3 * kFusedBatch) (&w.ev[0][0])[lane] = make_float2(0.f, 0.f);
-        if (lane == 0) w.changed = 0u;
+        if (lane == 0) w.changed = w.lists = 0u;
         __syncwarp();
         for (; cell < a.n_cells && nb < kFusedBatch; cell += nwarps, ++nb) {
             const int nt = a.ion.count[cell], t0 = a.ion.start[cell], mat = a.mat_of_cell[cell];
@@ -2385,6 +2481,7 @@ __global__ void __launch_bounds__(kBatchedThreads, 3) fused_cell_kernel(const __
         if (lane == 0) staged[wid] = nq;
         __syncthreads();
         fused_drain_block(&a, work, staged, &bacc);
+        fused_lists_block(&a, &F, work, &bacc);
         __syncthreads();
         for (unsigned ch = w.changed; ch; ch &= ch - 1u) {
             const int b = (__ffs(ch) - 1) >> 2;
@@ -2667,13 +2764,18 @@ static bool use_fused(const pcc_ctx* ctx, int n_cells, int precision, bool split
 }
 
 template <bool COMMIT>
-static void launch_fused(pcc_ctx* ctx, const StepArgs& a, unsigned run, cudaStream_t st)
+static void launch_fused(pcc_ctx* ctx, const StepArgs& a, unsigned run, const int (&cap)[3], int cap_ion, cudaStream_t st)
 {
     FusedArgs F;
-    for (int g = 0; g < 3; ++g)
-        for (int i = 0; i < 4; ++i) F.thr[g][i] = ctx->scan_thr[g][i];
     F.run = run;
-    F.qb = (uint32_t*)ctx->queue_b;
+    uint32_t* flat = (uint32_t*)ctx->queue_a;
+    for (int g = 0; g < 3; ++g) {
+        for (int i = 0; i < 4; ++i) F.thr[g][i] = ctx->scan_thr[g][i];
+        F.flat[g] = flat;
+        flat += cap[g];
+        F.qb[g] = (uint32_t*)ctx->queue_b + (size_t)g * cap_ion;
+        F.cap[g] = (uint32_t)cap[g];
+    }
     const int g = std::min(persistent_grid(ctx, (const void*)fused_cell_kernel<COMMIT>, 0, 0),
                            (a.n_cells + kFusedWarps - 1) / kFusedWarps);
     fused_cell_kernel<COMMIT><<<g, kBatchedThreads, 0, st>>>(a, F);
@@ -2695,7 +2797,9 @@ int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em,
     if (use_fused(ctx, cells->n_cells, precision, split)) {
         persistent_grid(ctx, (const void*)fused_cell_kernel<false>, 0, 0);
         persistent_grid(ctx, (const void*)fused_cell_kernel<true>, 0, 0);
-        return ensure_queue(ctx, 0, std::max<size_t>((size_t)ion->capacity, 1));
+        // a place for every projectile and, per group, for every target (see FusedArgs)
+        const size_t slots = (size_t)em->capacity + (size_t)ep->capacity + (size_t)ph->capacity;
+        return ensure_queue(ctx, slots / 2 + 1, std::max<size_t>(3 * (size_t)ion->capacity, 1));
     }
     int rc = ensure_lists(ctx, cells->n_cells);
     if (rc) return rc;
@@ -2810,8 +2914,9 @@ int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_sp
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_fail(e, "pcc_collide: launch");
             const unsigned run_bits = (run_em ? 1u : 0u) | (run_ep ? 2u : 0u) | (run_ph ? 4u : 0u);
-            if (committed) launch_fused<true>(ctx, a, run_bits, st);
-            else if (run_bits) launch_fused<false>(ctx, a, run_bits, st);
+            const int cap[3] = {em->capacity, ep->capacity, ph->capacity};
+            if (committed) launch_fused<true>(ctx, a, run_bits, cap, ion->capacity, st);
+            else if (run_bits) launch_fused<false>(ctx, a, run_bits, cap, ion->capacity, st);
             if (committed) *committed = true;
             e = cudaGetLastError();
             return e == cudaSuccess ? PCC_OK : cuda_fail(e, "pcc_collide: launch");
