@@ -753,6 +753,104 @@ __device__ void plain_ei_cell(const CtaGroup& grp, PlainShared& S, const StepArg
     block_acc_flush(S.acc, a.st);
 }
 
+// Puts the r largest ids of the a records from slot b on at their end, in order.
+// One warp; r passes for the largest of the rest.  (The whole list is ordered at
+// its commit; ordering it here, by one lane, took 1 ms for a cell of 1300.)
+__device__ void largest_last(const SpeciesView& P, int b, int a, int r, int lane)
+{
+    for (int last = a - 1; last > 0 && a - last <= r; --last) {   // warp-uniform
+        uint64_t top = 0;
+        int at = 0;
+#pragma unroll 4
+        for (int i = lane; i <= last; i += 32) {
+            const uint64_t id = P.pid[b + i];
+            if (id >= top) { top = id; at = i; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const uint64_t id = __shfl_xor_sync(0xffffffffu, top, o);
+            const int i = __shfl_xor_sync(0xffffffffu, at, o);
+            if (id > top || (id == top && i > at)) { top = id; at = i; }
+        }
+        if (lane == 0 && at != last) {
+            const int p = b + at, q = b + last;
+            const auto swap = [&](auto* v) { const auto t = v[p]; v[p] = v[q]; v[q] = t; };
+            swap(P.ux); swap(P.uy); swap(P.uz); swap(P.w); swap(P.pid);
+            if (P.x) swap(P.x);
+        }
+        __syncwarp();
+    }
+}
+
+// Stable removal of the absorbed photons (weight 0) from the first Np slots
+// of a cell region, keeping the order of the rest (including the Np..n_all
+// secondaries appended in this step), one warp.  The slots that the move vacates
+// keep copies of the last secondaries, which would be those that happened to
+// arrive last: the largest ids are put there first (see largest_last).  The
+// records before the first removed one are not touched; from there each batch
+// of 4 x 32 records is read into registers before any of it is written, and
+// destinations never pass sources.
+__device__ void compact_region_warp(const SpeciesView& P, int cell)
+{
+    constexpr unsigned kFull = 0xffffffffu;
+    constexpr int kU = 4;   // 32-record chunks loaded before any of them is stored
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const int p0 = P.start[cell], Np = P.count[cell];
+    const int n_all = Np + P.added[cell];
+    const bool has_x = P.x != nullptr;
+    // the records before the first removed one stay where they are
+    int c0 = 0;
+    for (; c0 < Np; c0 += 32 * kU) {
+        bool hole = false;
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int i = c0 + 32 * u + lane;
+            if (i < Np) hole |= P.w[p0 + i] == 0.f;
+        }
+        if (__any_sync(kFull, hole)) break;
+    }
+    if (c0 >= Np) return;   // nothing removed
+    int removed = 0;
+    for (int i = c0 + lane; i < Np; i += 32) removed += P.w[p0 + i] == 0.f ? 1 : 0;
+    largest_last(P, p0 + Np, n_all - Np, warp_sum(removed), lane);
+    int wr = c0;            // warp-uniform write position
+    for (int b = c0; b < n_all; b += 32 * kU) {
+        float ux[kU], uy[kU], uz[kU], w[kU], x[kU];
+        uint64_t pid[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int i = b + 32 * u + lane;
+            ux[u] = uy[u] = uz[u] = w[u] = x[u] = 0.f;
+            pid[u] = 0;
+            if (i < n_all) {
+                const int src = p0 + i;
+                ux[u] = P.ux[src]; uy[u] = P.uy[src]; uz[u] = P.uz[src]; w[u] = P.w[src];
+                if (has_x) x[u] = P.x[src];
+                pid[u] = P.pid[src];
+            }
+        }
+        __syncwarp();   // every record of the batch is read before any is overwritten
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int i = b + 32 * u + lane;
+            const bool keep = i < n_all && !(i < Np && w[u] == 0.f);
+            const unsigned m = __ballot_sync(kFull, keep);
+            if (keep) {
+                const int dst = p0 + wr + __popc(m & below);
+                if (dst != p0 + i) {
+                    P.ux[dst] = ux[u]; P.uy[dst] = uy[u]; P.uz[dst] = uz[u]; P.w[dst] = w[u];
+                    if (has_x) P.x[dst] = x[u];
+                    P.pid[dst] = pid[u];
+                }
+            }
+            wr += __popc(m);
+        }
+        __syncwarp();
+    }
+    if (lane == 0) P.count[cell] = wr - P.added[cell];
+}
+
 // Evaluates one photon - ion pair in full: 1 absorbed (weight set to 0), 0 not,
 // -1 the photon's momentum is not finite (flagged).
 __device__ __noinline__ int plain_bh_pair(const StepArgs* ap, const PlainCell* cp, uint32_t s, uint32_t j, uint32_t tau,
@@ -841,23 +939,7 @@ __device__ void plain_bh_cell(const CtaGroup& grp, PlainShared& S, const StepArg
                 *L = make_float4(v.x, v.y, k2.s, k2.c);
             }
         }
-        if (threadIdx.x == 0) {   // stable compaction of the region (rare path), see compact_region_warp
-            const bool has_x = P.x != nullptr;
-            const int Np = (int)c.Np, p0 = c.p0, n_all = Np + order_added(P, cell);
-            int wr = 0, removed = 0;
-            for (int i = 0; i < n_all; ++i) {
-                const int src = p0 + i;
-                if (i < Np && P.w[src] == 0.f) { ++removed; continue; }
-                if (wr != i) {
-                    const int dst = p0 + wr;
-                    P.ux[dst] = P.ux[src]; P.uy[dst] = P.uy[src]; P.uz[dst] = P.uz[src]; P.w[dst] = P.w[src];
-                    if (has_x) P.x[dst] = P.x[src];
-                    P.pid[dst] = P.pid[src];
-                }
-                ++wr;
-            }
-            P.count[cell] = Np - removed;
-        }
+        if (threadIdx.x < 32) compact_region_warp(P, cell);
     }
     __syncthreads();
     block_acc_flush(S.acc, a.st);
@@ -1923,74 +2005,6 @@ __global__ void __launch_bounds__(kBatchedThreads, 2) caseb_cand_kernel(const __
         __syncwarp();
     }
     fold_acc(acc, bacc, a.st);
-}
-
-// Stable removal of the absorbed photons (weight 0) from the first Np slots
-// of a cell region, keeping the order of the rest (including the Np..n_all
-// secondaries appended in this step), one warp.  The secondaries are put in
-// pid order first: the slots that the move vacates keep copies of the last of
-// them, which would otherwise be those that happened to arrive last.  The
-// records before the first removed one are not touched; from there each batch
-// of 4 x 32 records is read into registers before any of it is written, and
-// destinations never pass sources.
-__device__ void compact_region_warp(const SpeciesView& P, int cell)
-{
-    constexpr unsigned kFull = 0xffffffffu;
-    constexpr int kU = 4;   // 32-record chunks loaded before any of them is stored
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
-    const int p0 = P.start[cell], Np = P.count[cell];
-    const int n_all = Np + P.added[cell];
-    const bool has_x = P.x != nullptr;
-    // the records before the first removed one stay where they are
-    int c0 = 0;
-    for (; c0 < Np; c0 += 32 * kU) {
-        bool hole = false;
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int i = c0 + 32 * u + lane;
-            if (i < Np) hole |= P.w[p0 + i] == 0.f;
-        }
-        if (__any_sync(kFull, hole)) break;
-    }
-    if (c0 >= Np) return;   // nothing removed
-    if (lane == 0) order_added(P, cell);
-    __syncwarp();
-    int wr = c0;            // warp-uniform write position
-    for (int b = c0; b < n_all; b += 32 * kU) {
-        float ux[kU], uy[kU], uz[kU], w[kU], x[kU];
-        uint64_t pid[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int i = b + 32 * u + lane;
-            ux[u] = uy[u] = uz[u] = w[u] = x[u] = 0.f;
-            pid[u] = 0;
-            if (i < n_all) {
-                const int src = p0 + i;
-                ux[u] = P.ux[src]; uy[u] = P.uy[src]; uz[u] = P.uz[src]; w[u] = P.w[src];
-                if (has_x) x[u] = P.x[src];
-                pid[u] = P.pid[src];
-            }
-        }
-        __syncwarp();   // every record of the batch is read before any is overwritten
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int i = b + 32 * u + lane;
-            const bool keep = i < n_all && !(i < Np && w[u] == 0.f);
-            const unsigned m = __ballot_sync(kFull, keep);
-            if (keep) {
-                const int dst = p0 + wr + __popc(m & below);
-                if (dst != p0 + i) {
-                    P.ux[dst] = ux[u]; P.uy[dst] = uy[u]; P.uz[dst] = uz[u]; P.w[dst] = w[u];
-                    if (has_x) P.x[dst] = x[u];
-                    P.pid[dst] = pid[u];
-                }
-            }
-            wr += __popc(m);
-        }
-        __syncwarp();
-    }
-    if (lane == 0) P.count[cell] = wr - P.added[cell];
 }
 
 // Cells with an event in this call: the Kahan update of the cell ledger

@@ -19,11 +19,11 @@ __host__ __device__ inline SpeciesView view_of(const pcc_species& s)
 }
 
 // Orders the records appended to cell c by pid (they arrive in the order of
-// atomics) and returns their number.
-__device__ __forceinline__ int order_added(const SpeciesView& sp, int c)
+// atomics) and makes them live.
+__device__ __forceinline__ void commit_cell(const SpeciesView& sp, int c)
 {
     const int a = sp.added[c];
-    if (a == 0) return 0;
+    if (a == 0) return;
     const int b = sp.start[c] + sp.count[c];
     for (int i = 1; i < a; ++i) {   // insertion sort of the (few) appended records
         const uint64_t kp = sp.pid[b + i];
@@ -43,14 +43,6 @@ __device__ __forceinline__ int order_added(const SpeciesView& sp, int c)
         sp.ux[b + j + 1] = vx; sp.uy[b + j + 1] = vy; sp.uz[b + j + 1] = vz; sp.w[b + j + 1] = vw;
         if (sp.x) sp.x[b + j + 1] = vxx;
     }
-    return a;
-}
-
-// Orders the records appended to cell c and makes them live.
-__device__ __forceinline__ void commit_cell(const SpeciesView& sp, int c)
-{
-    const int a = order_added(sp, c);
-    if (a == 0) return;
     sp.count[c] += a;
     sp.added[c] = 0;
 }
