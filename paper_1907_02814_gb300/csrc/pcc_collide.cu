@@ -979,18 +979,26 @@ struct CellList {
 
 // Calls of kFusedMinCells cells up to kFusedCellsPerWarp for each resident warp
 // (24 on an SM: 18240 cells on 152 SMs) run as one kernel, a warp per cell (see
-// fused_cell_kernel).  Step in a graph, one kernel against the general sequence:
+// fused_cell_kernel), unless the step is long (below).  Step in a graph, one kernel against the general sequence:
 // 64 cells 10-18 against 87-102 us; 16384 cells of 64 to 256 electrons 47-75
 // against 103-118 us, log-normal ones 65-89 against 120-136 us; at 32768 cells
 // 84-152 against 109-148 us and for log-normal ones 122-179 against 131-165 us,
 // since the large cells, which the general scan takes first, hold up a warp.
-// Steps so long that large cells collide on most pairs take the longest on one
+// Steps so long that large cells collide on many pairs take the longest on one
 // warp, so its block works off long candidate lists together (see
 // fused_lists_block): 16384 log-normal cells with as many ions as electrons at
-// 1 fs 445 -> 265 us, the general sequence 277.
+// 1 fs 445 -> 265 us, the general sequence 277.  Where a block is not enough, the
+// general sequence spreads them over the chip, so that beyond a cell for every other
+// SM the step's largest x = n_i sigma beta c dt (pcc_ctx::pair_rate; solid Cu 0.0026
+// a fs) decides.  One kernel against the sequence, log-normal cells, us:
+//   64 cells at 300 fs 68/138; 152 cells at 30 fs 122/150 and 175/162, at 300 fs 189/165;
+//   2432 cells at 2.7 fs 60/154 and 195/191;
+//   16384 cells at 1.6 fs 120/189 and 296/279, at 2.7 fs 138/195 and 347/292
+// (the second pair with as many ions as electrons, the heaviest of the laws).
 constexpr int kFusedMinCells = 32;
 constexpr int kFusedCellsPerWarp = 5;
 constexpr int kFusedWarpsPerSM = 24;
+constexpr double kFusedX[3] = {0.1, 0.007, 0.0043};   // up to one cell per SM, up to 16, and above
 constexpr int kClassBlock = 1024;                 // cells per class-sort block
 
 // Class of a cell with N_pair = max(N_p, N_t) pairs: with b the bit length
@@ -2071,6 +2079,7 @@ struct FusedArgs {
     // [target capacity] of the others.
     uint32_t *flat[3], *qb[3];
     uint32_t cap[3];    // projectile capacities
+    int warps;          // warps of a block that take cells
 };
 
 constexpr int kFusedWarps = kBatchedThreads / 32;
@@ -2465,9 +2474,9 @@ __global__ void __launch_bounds__(kBatchedThreads, 3) fused_cell_kernel(const __
     __syncthreads();
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     FusedWarp& w = work[wid];
-    const int nwarps = gridDim.x * kFusedWarps;
-    int cell = blockIdx.x * kFusedWarps + wid;
-    for (int lead = blockIdx.x * kFusedWarps; lead < a.n_cells; lead += kFusedBatch * nwarps) {   // lead: warp 0's cell
+    const int nwarps = gridDim.x * F.warps;
+    int cell = wid < F.warps ? blockIdx.x * F.warps + wid : a.n_cells;
+    for (int lead = blockIdx.x * F.warps; lead < a.n_cells; lead += kFusedBatch * nwarps) {   // lead: warp 0's cell
         const int first = cell;
         int nq = 0, nb = 0;
         if (lane < 3 * kFusedBatch) (&w.ev[0][0])[lane] = make_float2(0.f, 0.f);
@@ -2771,10 +2780,12 @@ static void warm_occupancy(pcc_ctx* ctx, int stage)
 // needs them apart, a context with its own wait limit asks for the staged
 // copies that the limit is about, and calls of a few cells keep the general
 // sequence, whose launch count callers can rely on.
-static bool use_fused(const pcc_ctx* ctx, int n_cells, int precision, bool split)
+static bool use_fused(const pcc_ctx* ctx, int n_cells, int precision, bool split, double dt)
 {
-    return precision == PCC_FP32_BATCHED && !split && n_cells >= kFusedMinCells &&
-           n_cells <= kFusedCellsPerWarp * kFusedWarpsPerSM * ctx->num_sms && ctx->wait_polls == kWaitPolls;
+    if (precision != PCC_FP32_BATCHED || split || ctx->wait_polls != kWaitPolls) return false;
+    if (n_cells < kFusedMinCells || n_cells > kFusedCellsPerWarp * kFusedWarpsPerSM * ctx->num_sms) return false;
+    if (2 * n_cells <= ctx->num_sms) return true;
+    return ctx->pair_rate * dt <= kFusedX[n_cells <= ctx->num_sms ? 0 : n_cells <= 16 * ctx->num_sms ? 1 : 2];
 }
 
 template <bool COMMIT>
@@ -2790,14 +2801,15 @@ static void launch_fused(pcc_ctx* ctx, const StepArgs& a, unsigned run, const in
         F.qb[g] = (uint32_t*)ctx->queue_b + (size_t)g * cap_ion;
         F.cap[g] = (uint32_t)cap[g];
     }
-    const int g = std::min(persistent_grid(ctx, (const void*)fused_cell_kernel<COMMIT>, 0, 0),
-                           (a.n_cells + kFusedWarps - 1) / kFusedWarps);
-    fused_cell_kernel<COMMIT><<<g, kBatchedThreads, 0, st>>>(a, F);
+    // few cells: spread over the SMs, so that more warps are there to work off long lists
+    const int grid = persistent_grid(ctx, (const void*)fused_cell_kernel<COMMIT>, 0, 0);
+    F.warps = std::min(kFusedWarps, (a.n_cells + grid - 1) / grid);
+    fused_cell_kernel<COMMIT><<<std::min(grid, (a.n_cells + F.warps - 1) / F.warps), kBatchedThreads, 0, st>>>(a, F);
     note_launches(1);
 }
 
 int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em, const pcc_species* ep,
-                    const pcc_species* ph, const pcc_species* ion, unsigned mask, int precision, bool split)
+                    const pcc_species* ph, const pcc_species* ion, double dt, unsigned mask, int precision, bool split)
 {
     if (!ctx || !cells || !em || !ep || !ph || !ion || cells->n_cells < 1) {
         set_error("pcc_collide: invalid argument");
@@ -2808,7 +2820,7 @@ int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em,
     const bool ei = (mask & (PCC_BREMS | PCC_TRIDENT)) != 0, bh = (mask & PCC_BH) != 0;
     const bool run_em = ei && (groups & PCC_GROUP_EM), run_ep = ei && (groups & PCC_GROUP_EP);
     const bool run_ph = bh && (groups & PCC_GROUP_PH);
-    if (use_fused(ctx, cells->n_cells, precision, split)) {
+    if (use_fused(ctx, cells->n_cells, precision, split, dt)) {
         persistent_grid(ctx, (const void*)fused_cell_kernel<false>, 0, 0);
         persistent_grid(ctx, (const void*)fused_cell_kernel<true>, 0, 0);
         // a place for every projectile and, per group, for every target (see FusedArgs)
@@ -2922,9 +2934,9 @@ int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_sp
     int stage = 0;
     if (precision == PCC_FP32_BATCHED) {
         const bool split = after_group != nullptr;
-        int rc = collide_prepare(ctx, cells, em, ep, ph, ion, mask, precision, split);
+        int rc = collide_prepare(ctx, cells, em, ep, ph, ion, dt, mask, precision, split);
         if (rc) return rc;
-        if (use_fused(ctx, cells->n_cells, precision, split)) {
+        if (use_fused(ctx, cells->n_cells, precision, split, dt)) {
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_fail(e, "pcc_collide: launch");
             const unsigned run_bits = (run_em ? 1u : 0u) | (run_ep ? 2u : 0u) | (run_ph ? 4u : 0u);

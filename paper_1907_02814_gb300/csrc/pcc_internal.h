@@ -32,6 +32,7 @@ struct pcc_ctx {
     float* f_tri_split_cdf = nullptr;
     float* f_Z = nullptr;             // [n_mat] nuclear charge as float
     float* f_bound = nullptr;         // [n_mat][3] acceptance bounds: Brems, Trident, BH
+    double pair_rate = 0.0;           // largest n_i sigma beta c of the materials [1/s] (Brems, BH), for the choice of kernels
     // status and counters
     pcc::DevStats* stats = nullptr;
     // scratch
@@ -120,7 +121,7 @@ TableGeom make_geom(const pcc_table_spec& s);
 // set up ahead (allocations, occupancy queries) so the call itself can be
 // captured into a graph.  split: the groups are wanted one by one.
 int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em, const pcc_species* ep,
-                    const pcc_species* ph, const pcc_species* ion, unsigned mask, int precision, bool split);
+                    const pcc_species* ph, const pcc_species* ion, double dt, unsigned mask, int precision, bool split);
 // The work of pcc_collide on stream st.  After the kernels of group g
 // (0 e-, 1 e+, 2 photons) are enqueued, whether or not the group runs,
 // after_group(user, g) is called if given, so that a caller can record

@@ -556,11 +556,17 @@ extern "C" int pcc_tables_build(pcc_ctx* ctx, const pcc_material* mats, int n_ma
     bounds_kernel<<<n_mats, 32, 0, st>>>(ctx->screen, ctx->brems_sigma, ctx->bh_sigma, g, n_mats,
                                                      ctx->f_bound);
     note_launches(13);
+    std::vector<float> bound(3 * M);
     e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(bound.data(), ctx->f_bound, bound.size() * sizeof(float), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFree(dmats);
     cudaFree(tfd);
     if (e != cudaSuccess) { free_tables(ctx); return cuda_fail(e, "pcc_tables_build: kernels"); }
+    ctx->pair_rate = 0.0;
+    for (size_t m = 0; m < M; ++m)   // the bounds hold twice the cross section, for ions that meet the projectile
+        ctx->pair_rate = std::max(ctx->pair_rate, 0.5 * kC * mats[m].n_i * std::max(bound[3 * m], bound[3 * m + 2]));
     ctx->n_mat = n_mats;
     ctx->spec = s;
     return PCC_OK;

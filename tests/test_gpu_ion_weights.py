@@ -16,7 +16,7 @@ SPEC = dict(n_rows=64, n_cols=64)
 
 
 def workload():
-    n, rng = 400, np.random.default_rng(17)
+    n, rng = 75, np.random.default_rng(17)
     wl = W.solid_cu(n_cells=n, e_per_cell=rng.integers(1, 500, n), i_per_cell=rng.integers(2, 9, n),
                     photons_per_cell=rng.integers(20, 400, n), seed=41, dt=2e-12, T_mev=30.0)
     wl.species["ep"] = W.solid_cu(n_cells=n, e_per_cell=rng.integers(20, 300, n), i_per_cell=1, seed=42, T_mev=30.0).species["em"]
