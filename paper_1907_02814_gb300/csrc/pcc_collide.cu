@@ -2775,6 +2775,11 @@ static void warm_occupancy(pcc_ctx* ctx, int stage)
     persistent_grid(ctx, (const void*)caseb_cand_kernel<GROUP>, stage, 0);
 }
 
+static bool fused_range(const pcc_ctx* ctx, int n_cells)
+{
+    return n_cells >= kFusedMinCells && n_cells <= kFusedCellsPerWarp * kFusedWarpsPerSM * ctx->num_sms;
+}
+
 // The fused kernel takes the call's cells whole: chosen where launches bound
 // the step (see kFusedCellsPerWarp).  A call with timing events between the groups
 // needs them apart, a context with its own wait limit asks for the staged
@@ -2783,7 +2788,7 @@ static void warm_occupancy(pcc_ctx* ctx, int stage)
 static bool use_fused(const pcc_ctx* ctx, int n_cells, int precision, bool split, double dt)
 {
     if (precision != PCC_FP32_BATCHED || split || ctx->wait_polls != kWaitPolls) return false;
-    if (n_cells < kFusedMinCells || n_cells > kFusedCellsPerWarp * kFusedWarpsPerSM * ctx->num_sms) return false;
+    if (!fused_range(ctx, n_cells)) return false;
     if (2 * n_cells <= ctx->num_sms) return true;
     return ctx->pair_rate * dt <= kFusedX[n_cells <= ctx->num_sms ? 0 : n_cells <= 16 * ctx->num_sms ? 1 : 2];
 }
@@ -2809,7 +2814,7 @@ static void launch_fused(pcc_ctx* ctx, const StepArgs& a, unsigned run, const in
 }
 
 int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em, const pcc_species* ep,
-                    const pcc_species* ph, const pcc_species* ion, double dt, unsigned mask, int precision, bool split)
+                    const pcc_species* ph, const pcc_species* ion, unsigned mask, int precision)
 {
     if (!ctx || !cells || !em || !ep || !ph || !ion || cells->n_cells < 1) {
         set_error("pcc_collide: invalid argument");
@@ -2820,20 +2825,24 @@ int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em,
     const bool ei = (mask & (PCC_BREMS | PCC_TRIDENT)) != 0, bh = (mask & PCC_BH) != 0;
     const bool run_em = ei && (groups & PCC_GROUP_EM), run_ep = ei && (groups & PCC_GROUP_EP);
     const bool run_ph = bh && (groups & PCC_GROUP_PH);
-    if (use_fused(ctx, cells->n_cells, precision, split, dt)) {
-        persistent_grid(ctx, (const void*)fused_cell_kernel<false>, 0, 0);
-        persistent_grid(ctx, (const void*)fused_cell_kernel<true>, 0, 0);
-        // a place for every projectile and, per group, for every target (see FusedArgs)
-        const size_t slots = (size_t)em->capacity + (size_t)ep->capacity + (size_t)ph->capacity;
-        return ensure_queue(ctx, slots / 2 + 1, std::max<size_t>(3 * (size_t)ion->capacity, 1));
-    }
+    // Whichever way this call goes, the buffers of both are made: a later call on
+    // the same cells may go the other way inside a caller's capture, where nothing
+    // can be allocated, and a graph captured one way keeps its buffers when a
+    // call goes the other.
     int rc = ensure_lists(ctx, cells->n_cells);
     if (rc) return rc;
-    size_t cap_a = 0;
+    size_t cap_a = 0, cap_b = (size_t)ion->capacity;
     if (run_em) cap_a = std::max(cap_a, (size_t)em->capacity);
     if (run_ep) cap_a = std::max(cap_a, (size_t)ep->capacity);
     if (run_ph) cap_a = std::max(cap_a, (size_t)ph->capacity);
-    rc = ensure_queue(ctx, std::max<size_t>(cap_a, 1), std::max<size_t>((size_t)ion->capacity, 1));
+    if (fused_range(ctx, cells->n_cells)) {
+        // a place for every projectile and, per group, for every target (see FusedArgs)
+        cap_a = std::max(cap_a, ((size_t)em->capacity + (size_t)ep->capacity + (size_t)ph->capacity) / 2 + 1);
+        cap_b *= 3;
+        persistent_grid(ctx, (const void*)fused_cell_kernel<false>, 0, 0);
+        persistent_grid(ctx, (const void*)fused_cell_kernel<true>, 0, 0);
+    }
+    rc = ensure_queue(ctx, std::max<size_t>(cap_a, 1), std::max<size_t>(cap_b, 1));
     if (rc) return rc;
     const int stage = table_stage_bytes(ctx);
     if (run_em) warm_occupancy<kGroupEm>(ctx, stage);
@@ -2934,7 +2943,7 @@ int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_sp
     int stage = 0;
     if (precision == PCC_FP32_BATCHED) {
         const bool split = after_group != nullptr;
-        int rc = collide_prepare(ctx, cells, em, ep, ph, ion, dt, mask, precision, split);
+        int rc = collide_prepare(ctx, cells, em, ep, ph, ion, mask, precision);
         if (rc) return rc;
         if (use_fused(ctx, cells->n_cells, precision, split, dt)) {
             cudaError_t e = cudaGetLastError();

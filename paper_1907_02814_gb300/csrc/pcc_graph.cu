@@ -73,8 +73,7 @@ extern "C" int pcc_steps_capture(pcc_ctx* ctx, const pcc_step_desc* d, uint64_t 
     }
     pcc_free_graph(ctx);
     // every allocation and occupancy query of the step happens here, outside the capture
-    int rc = collide_prepare(ctx, d->cells, d->em, d->ep, d->ph, d->ion, d->dt, d->mask, d->precision,
-                             timing != 0);
+    int rc = collide_prepare(ctx, d->cells, d->em, d->ep, d->ph, d->ion, d->mask, d->precision);
     if (rc) return rc;
     cudaError_t e = cudaSuccess;
     if (!ctx->capture_stream) e = cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking);

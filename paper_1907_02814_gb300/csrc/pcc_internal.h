@@ -119,9 +119,9 @@ TableGeom make_geom(const pcc_table_spec& s);
 
 // Buffers and launch geometry of a pcc_collide call with these arguments,
 // set up ahead (allocations, occupancy queries) so the call itself can be
-// captured into a graph.  split: the groups are wanted one by one.
+// captured into a graph.
 int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em, const pcc_species* ep,
-                    const pcc_species* ph, const pcc_species* ion, double dt, unsigned mask, int precision, bool split);
+                    const pcc_species* ph, const pcc_species* ion, unsigned mask, int precision);
 // The work of pcc_collide on stream st.  After the kernels of group g
 // (0 e-, 1 e+, 2 photons) are enqueued, whether or not the group runs,
 // after_group(user, g) is called if given, so that a caller can record
