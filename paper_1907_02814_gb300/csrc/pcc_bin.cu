@@ -838,8 +838,8 @@ extern "C" int pcc_totals(pcc_ctx* ctx, int n_cells, const pcc_species* sp, int 
 {
     if (!ctx || !sp || !out || n_cells < 1) { set_error("pcc_totals: invalid argument"); return PCC_E_INVALID; }
     // four resident blocks per SM, fewer where the cells do not fill them
-    const int blocks = std::min(4 * std::max(ctx->num_sms, 1), (n_cells + 7) / 8);
-    int rc = ensure_scratch(ctx, (size_t)blocks * 3 * sizeof(double));
+    const int most = 4 * std::max(ctx->num_sms, 1), blocks = std::min(most, (n_cells + 7) / 8);
+    int rc = ensure_scratch(ctx, (size_t)most * 3 * sizeof(double));   // the same for every call, also in a later capture
     if (rc) return rc;
     double* partial = (double*)ctx->scratch;
     cudaStream_t st = (cudaStream_t)stream;

@@ -80,6 +80,20 @@ def test_collide_captured_after_the_other_way(pcc, how):
     ref.close()
 
 
+def test_totals_captured_on_more_cells(pcc):
+    ctx, ctx2 = context(pcc), context(pcc)
+    _, small, _ = cells(pcc, ctx2, 8)                       # binned elsewhere: this context has no scratch yet
+    _, big, _ = cells(pcc, ctx2, 4000)
+    pcc.totals(ctx, 8, small["em"])
+    out = []
+    g = capture(lambda: out.append(pcc.totals(ctx, 4000, big["em"])))
+    g.replay()
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(out[0].cpu().numpy(), pcc.totals(ctx2, 4000, big["em"]).cpu().numpy())
+    ctx.close()
+    ctx2.close()
+
+
 def test_chained_kernels_after_a_join(pcc):
     """The captured stream has just joined another one, so that the first kernel depends on two."""
     ctx, ref = context(pcc), context(pcc)
