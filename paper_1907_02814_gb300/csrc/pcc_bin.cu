@@ -740,7 +740,10 @@ extern "C" int pcc_bin(pcc_ctx* ctx, const pcc_particles* in, int n_cells, pcc_s
     }
     cudaStream_t st = (cudaStream_t)stream;
     const int n = in->n, nb = (n_cells + kScanBlock - 1) / kScanBlock;
-    // scratch: counts with the class counters, offsets, cursors, block sums, totals, class lists, records
+    // scratch: counts with the class counters, offsets, cursors, block sums, totals,
+    // class lists, records.  Its size goes by the capacity, not by the particles, so
+    // that a run whose species grow allocates once and what a captured graph holds
+    // of it stays; only where memory is too short for that, by the particles.
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~size_t(255); return o; };
     const size_t o_counts = take(((size_t)n_cells + kSortClasses) * sizeof(int));
@@ -749,11 +752,13 @@ extern "C" int pcc_bin(pcc_ctx* ctx, const pcc_particles* in, int n_cells, pcc_s
     const size_t o_sums = take(nb * sizeof(BlockSums));
     const size_t o_tot = take(sizeof(BinTotals));
     size_t o_list[kSortClasses];
-    // cells of a class hold at least so many particles each
-    const int at_least[kSortClasses] = {kSortWarpCap + 1, kSortCap0 + 1, kSortCap1 + 1};
-    for (int k = 0; k < kSortClasses; ++k) o_list[k] = take((size_t)std::min(n_cells, n / at_least[k] + 1) * sizeof(int));
-    const size_t o_tmp = take((size_t)n * sizeof(TmpRec));
-    int rc = ensure_scratch(ctx, off);
+    for (int k = 0; k < kSortClasses; ++k) o_list[k] = take((size_t)n_cells * sizeof(int));
+    const size_t o_tmp = off, cap = (size_t)out->capacity;
+    int rc = ensure_scratch(ctx, o_tmp + cap * sizeof(TmpRec));
+    if (rc && (size_t)n < cap) {
+        cudaGetLastError();
+        rc = ensure_scratch(ctx, o_tmp + (size_t)n * sizeof(TmpRec));
+    }
     if (rc) return rc;
     rc = ensure_bin_host(ctx);
     if (rc) return rc;

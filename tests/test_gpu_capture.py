@@ -141,3 +141,21 @@ def test_graph_keeps_its_buffers_when_a_call_goes_the_other_way(pcc):
     status, stats = ctx.read_status()
     assert not status & pcc.ST_CAPACITY and sum(stats["created"]) > 0
     ctx.close()
+
+
+def test_binning_a_growing_species_allocates_once(pcc):
+    ctx = context(pcc)
+    n_cells, cap = 500, 4_000_000
+    sp = pcc.DeviceSpecies.empty(n_cells, cap)
+    rng = np.random.default_rng(2)
+    parts = []
+    for n in (1000, 200_000, 1_000_000, 2_500_000):
+        f = rng.normal(size=n).astype(np.float32)
+        parts.append(pcc.particles_to_device({"ux": f, "uy": f, "uz": f, "w": np.ones(n, np.float32), "x": None,
+                                              "pid": np.arange(n, dtype=np.uint64), "cell": rng.integers(0, n_cells, n).astype(np.int32)}))
+    pcc.bin(ctx, parts[0], n_cells, sp, slack_abs=1, slack_rel=0.0)
+    before = used()
+    for p in parts[1:]:
+        pcc.bin(ctx, p, n_cells, sp, slack_abs=1, slack_rel=0.0)
+        assert used() == before
+    ctx.close()
