@@ -231,8 +231,9 @@ int pcc_collide(pcc_ctx *ctx, const pcc_cells *cells, pcc_species *em, pcc_speci
  * of 16 to 2 lanes for each smaller one; min_blocks_per_sm
  * (2 to 6) selects the register budget of the kernel (a minimum of that
  * many resident 256-thread blocks per SM) and blocks_per_sm caps the
- * persistent grid (0 = as many as fit).  Applies to later pcc_collide calls
- * on this context.  PCC_E_INVALID outside these ranges. */
+ * persistent grid (0 = as many as fit).  Calls that run as one kernel (see
+ * pcc_set_wait_limit) take the cap; their register budget is fixed.  Applies to
+ * later pcc_collide calls on this context.  PCC_E_INVALID outside these ranges. */
 int pcc_set_schedule(pcc_ctx *ctx, int min_blocks_per_sm, int blocks_per_sm);
 
 /* Lane groups of the batched scan (no counterpart in the paper; a
@@ -334,7 +335,8 @@ int pcc_totals_noalloc(int n_cells, const pcc_species *sp, int is_photon, double
  * timing != 0 adds five timing events per step (before the e- group, after
  * each group, after the commits), read by pcc_steps_timing; on the batched
  * path the size-class sort of all groups runs before the e- group's kernels
- * and is timed with them.
+ * and is timed with them.  Its groups run apart, also where a graph without
+ * timing runs each step as one kernel: same results, another time.
  * pcc_steps_launch enqueues the whole graph on the stream.  A launch
  * repeats the same step indices: capture again to go on. */
 typedef struct {

@@ -2807,7 +2807,7 @@ static void launch_fused(pcc_ctx* ctx, const StepArgs& a, unsigned run, const in
         F.cap[g] = (uint32_t)cap[g];
     }
     // few cells: spread over the SMs, so that more warps are there to work off long lists
-    const int grid = persistent_grid(ctx, (const void*)fused_cell_kernel<COMMIT>, 0, 0);
+    const int grid = persistent_grid(ctx, (const void*)fused_cell_kernel<COMMIT>, 0, ctx->blocks_per_sm);
     F.warps = std::min(kFusedWarps, (a.n_cells + grid - 1) / grid);
     fused_cell_kernel<COMMIT><<<std::min(grid, (a.n_cells + F.warps - 1) / F.warps), kBatchedThreads, 0, st>>>(a, F);
     note_launches(1);

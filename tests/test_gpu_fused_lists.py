@@ -86,6 +86,35 @@ def test_long_lists(pcc, law, n_cells, graph):
             assert np.array_equal(a[k][f], b[k][f]), (k, f)
 
 
+@pytest.mark.parametrize("blocks_per_sm", [1, 2])
+def test_grid_cap(pcc, blocks_per_sm):
+    """pcc_set_schedule's cap on the grid: warps take more cells each, in several batches; the same bits."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 8 * 8 * sms + 77                            # more than a batch of eight cells for each warp of one block per SM
+    wl = W.solid_cu(n_cells=n, e_per_cell=30, i_per_cell=7, photons_per_cell=9, seed=3, dt=1e-15, T_mev=20.0)
+    out = []
+    for cap in (0, blocks_per_sm):
+        ctx = pcc.Context(0)
+        ctx.tables_build([pcc.material(29, 5.0, 8.5e28, 100.0)], pcc.table_spec(n_rows=63, n_cols=65))
+        ctx.set_schedule(4, cap)
+        dev = {}
+        for name, d in wl.species.items():
+            dev[name] = pcc.DeviceSpecies.empty(n, len(d["w"]) + 31 * n)
+            pcc.bin(ctx, pcc.particles_to_device(d), n, dev[name], slack_abs=30, slack_rel=0.0)
+        mat = torch.zeros(n, dtype=torch.int32, device="cuda")
+        n0 = pcc.launch_count()
+        ctx.steps_capture(n, mat, wl.ion_mass, dev["em"], dev["ep"], dev["ph"], dev["ion"], wl.dt, 5, 0, 3)
+        ctx.steps_launch()
+        _, stats = ctx.read_status()
+        assert pcc.launch_count() - n0 == 3 and stats["created"][0] > 50
+        out.append((stats, {k: [getattr(dev[k], f) for f in FIELDS if f != "x"] for k in ("em", "ep", "ph")}))
+        ctx.close()
+    for f in ("pairs", "accepted", "created", "candidates"):
+        assert out[0][0][f] == out[1][0][f]
+    for k in ("em", "ep", "ph"):
+        assert all(torch.equal(x, y) for x, y in zip(out[0][1][k], out[1][1][k])), k
+
+
 def test_slots_beyond_a_staged_candidate(pcc):
     """A cell of 2^27 + 2^25 electrons: the same electrons change on both paths."""
     n_cells, big = 33, (1 << 27) + (1 << 25)
