@@ -35,6 +35,7 @@ struct StepArgs {
     PhiloxKeys keys;         // round keys of the seed
     float f_cdt;             // c dt in float
     int wait_polls;          // bounded waits give up after this many polls
+    int thr[2][4];           // scan lane groups of the e- and e+ groups (see CellList)
 };
 
 // ---- per-thread accumulators ---------------------------------------------
@@ -782,16 +783,92 @@ __device__ void largest_last(const SpeciesView& P, int b, int a, int r, int lane
     }
 }
 
+__device__ __forceinline__ PermKeys perm_keys(const StepArgs& a, int group, int cell)
+{
+    const Philox4 kp = draw_k(0, (uint32_t)cell, (uint32_t)a.step, stream_tag(group, kPerm, 0), a.keys);
+    return PermKeys{{kp.v[0], kp.v[1], kp.v[2], kp.v[3]}};
+}
+
+__device__ __forceinline__ int size_class(int np, int nt);
+
+// Places pair j of group g (e- or e+) of a cell in the order in which its candidates
+// are taken up when nothing overtakes: the order in which the scan's lane group marks
+// them, on the FP64 path (plain) that of the slots.  All 32 lanes, a pair each.
+__device__ __forceinline__ uint32_t pair_order(const StepArgs& a, int g, int cell, uint32_t j, bool plain, int lane)
+{
+    constexpr uint32_t S = 4;   // slots per draw (see AcceptSlots), 32 / S draws per candidate mask
+    const uint32_t Np = (uint32_t)(g ? a.ep : a.em).count[cell], Nt = (uint32_t)a.ion.count[cell], NL = max(Np, Nt);
+    if (Np == 0 || Nt == 0) return j;
+    const int cls = size_class((int)Np, (int)Nt);
+    const int* thr = a.thr[g];
+    const uint32_t G = cls >= thr[0] ? 32 : cls >= thr[1] ? 16 : cls >= thr[2] ? 8 : cls >= thr[3] ? 4 : 2;
+    j %= NL;
+    if (Np < Nt) {   // units of a draw, G at a time; of each unit's pairs the first of all lanes first
+        const uint32_t m = j / Np, s = j - m * Np, i = m * ((Np + S - 1) / S) + s / S;
+        return plain ? j : (i / G * S + s % S) * G + i % G;
+    }
+    const PermKeys rk = perm_keys(a, g, cell);
+    uint32_t s = 0;
+    if (NL <= 32) {
+        const uint32_t r = perm_pos_small(min((uint32_t)lane, NL - 1u), NL, rk);
+        for (uint32_t q = 0; q < NL; ++q)
+            if (__shfl_sync(0xffffffffu, r, (int)q) == j) s = q;
+    } else {
+        s = perm_elem_large(j, NL, rk);
+    }
+    const uint32_t it = s / (S * G), gl = s / S % G;
+    return plain ? s : ((it / (32 / S) * G + gl) * (32 / S) + it % (32 / S)) * S + s % S;
+}
+
+// Orders the photons appended to a cell (n of them from slot b on) so that the last
+// r, copies of which stay behind when they are moved down by r, do not depend on the
+// order of atomics: in pair_order, e- before e+, which is how they mostly arrive; of
+// long lists the largest ids come last.  All 32 lanes.
+__device__ __noinline__ void order_added(const StepArgs* ap, int cell, int b, int n, int r, bool plain)
+{
+    constexpr unsigned kFull = 0xffffffffu;
+    const SpeciesView& P = ap->ph;
+    const int lane = threadIdx.x & 31;
+    if (n < 2) return;
+    if (n > 32) { largest_last(P, b, n, r, lane); return; }
+    const int sl = b + min(lane, n - 1);
+    const uint64_t id = P.pid[sl];
+    const bool ep = (id >> 41 & 7u) == kChBremsEp;
+    const uint32_t j = (uint32_t)(id >> 1) & 0xFFFFu;
+    uint32_t key = 0;
+    for (int g = 0; g < 2; ++g) {
+        const uint32_t k = pair_order(*ap, g, cell, j, plain, lane);
+        if (ep == (g == 1)) key = k;
+    }
+    int rank = 0;
+    for (int q = 0; q < n; ++q) {
+        const bool e2 = __shfl_sync(kFull, (int)ep, q) != 0;
+        const uint32_t k2 = __shfl_sync(kFull, key, q);
+        const uint64_t i2 = __shfl_sync(kFull, id, q);
+        rank += e2 != ep ? ep : k2 < key || (k2 == key && i2 < id);
+    }
+    const float ux = P.ux[sl], uy = P.uy[sl], uz = P.uz[sl], w = P.w[sl], x = P.x ? P.x[sl] : 0.f;
+    __syncwarp();
+    if (lane < n) {
+        const int to = b + rank;
+        P.ux[to] = ux; P.uy[to] = uy; P.uz[to] = uz; P.w[to] = w;
+        if (P.x) P.x[to] = x;
+        P.pid[to] = id;
+    }
+    __syncwarp();
+}
+
 // Stable removal of the absorbed photons (weight 0) from the first Np slots
 // of a cell region, keeping the order of the rest (including the Np..n_all
 // secondaries appended in this step), one warp.  The slots that the move vacates
 // keep copies of the last secondaries, which would be those that happened to
-// arrive last: the largest ids are put there first (see largest_last).  The
+// arrive last, so they are ordered first (see order_added).  The
 // records before the first removed one are not touched; from there each batch
 // of 4 x 32 records is read into registers before any of it is written, and
 // destinations never pass sources.
-__device__ void compact_region_warp(const SpeciesView& P, int cell)
+__device__ void compact_region_warp(const StepArgs& a, int cell, bool plain)
 {
+    const SpeciesView& P = a.ph;
     constexpr unsigned kFull = 0xffffffffu;
     constexpr int kU = 4;   // 32-record chunks loaded before any of them is stored
     const int lane = threadIdx.x & 31;
@@ -813,7 +890,7 @@ __device__ void compact_region_warp(const SpeciesView& P, int cell)
     if (c0 >= Np) return;   // nothing removed
     int removed = 0;
     for (int i = c0 + lane; i < Np; i += 32) removed += P.w[p0 + i] == 0.f ? 1 : 0;
-    largest_last(P, p0 + Np, n_all - Np, warp_sum(removed), lane);
+    order_added(&a, cell, p0 + Np, n_all - Np, warp_sum(removed), plain);
     int wr = c0;            // warp-uniform write position
     for (int b = c0; b < n_all; b += 32 * kU) {
         float ux[kU], uy[kU], uz[kU], w[kU], x[kU];
@@ -939,7 +1016,7 @@ __device__ void plain_bh_cell(const CtaGroup& grp, PlainShared& S, const StepArg
                 *L = make_float4(v.x, v.y, k2.s, k2.c);
             }
         }
-        if (threadIdx.x < 32) compact_region_warp(P, cell);
+        if (threadIdx.x < 32) compact_region_warp(a, cell, true);
     }
     __syncthreads();
     block_acc_flush(S.acc, a.st);
@@ -1879,12 +1956,6 @@ __device__ __forceinline__ bool eval_pair(const StepArgs& a, const Tab<float>& t
     return event;
 }
 
-__device__ __forceinline__ PermKeys perm_keys(const StepArgs& a, int group, int cell)
-{
-    const Philox4 kp = draw_k(0, (uint32_t)cell, (uint32_t)a.step, stream_tag(group, kPerm, 0), a.keys);
-    return PermKeys{{kp.v[0], kp.v[1], kp.v[2], kp.v[3]}};
-}
-
 // A candidate of a cell with N_p >= N_t (one pair per projectile slot s).
 template <bool PH>
 __device__ __forceinline__ bool flat_pair(const StepArgs& a, const Tab<float>& tb, int group, int cell, const CellRec& cm,
@@ -2052,7 +2123,7 @@ __global__ void finalize_kernel(const __grid_constant__ StepArgs a, Queue Q)
         const int cell = Q.flagged[kk];
         if (cell < 0 || cell >= a.n_cells) continue;
         if (lane == 0) finalize_ledger(a, Q, cell);
-        compact_region_warp(a.ph, cell);
+        compact_region_warp(a, cell, false);
         __syncwarp();
         if (lane == 0) Q.flag[cell] = 0;
     }
@@ -2253,7 +2324,7 @@ __device__ __noinline__ void fused_finish(const StepArgs* ap, FusedWarp* w, int 
         *Lg = make_float4(ka.s, ka.c, kb.s, kb.c);
     }
     __syncwarp();
-    if (ch >> kGroupPh & 1u) compact_region_warp(a.ph, cell);
+    if (ch >> kGroupPh & 1u) compact_region_warp(a, cell, false);
     __syncwarp();
 }
 
@@ -2587,6 +2658,8 @@ static StepArgs make_args(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em,
     a.keys = philox_keys(seed);
     a.f_cdt = (float)(kC * dt);
     a.wait_polls = ctx->wait_polls;
+    for (int g = 0; g < 2; ++g)
+        for (int i = 0; i < 4; ++i) a.thr[g][i] = ctx->scan_thr[g][i];
     a.st = ctx->stats;
     return a;
 }
