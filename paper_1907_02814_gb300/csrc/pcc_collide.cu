@@ -2573,9 +2573,9 @@ __global__ void __launch_bounds__(kBatchedThreads, 3) fused_cell_kernel(const __
             if (ng > 0) fused_scan<kGroupPh>(a, F, w, nb, cell, g0, ng, t0, nt, mat, is, nq, lane, bacc);
         }
         if (lane == 0) staged[wid] = nq;
-        __syncthreads();
+        const int some = __syncthreads_or(lane == 0 && w.lists);
         fused_drain_block(&a, work, staged, &bacc);
-        fused_lists_block(&a, &F, work, &bacc);
+        if (some) fused_lists_block(&a, &F, work, &bacc);
         __syncthreads();
         for (unsigned ch = w.changed; ch; ch &= ch - 1u) {
             const int b = (__ffs(ch) - 1) >> 2;
