@@ -260,7 +260,7 @@ int pcc_get_scan_classes(const pcc_ctx *ctx, int group, int *thresholds);
  * a second bounded wait that lets the copy land.  polls = 0 makes every
  * staged launch time out, to test the status path without a hang or a
  * fault.  (A context with its own limit takes the launch sequence with the
- * staged copies at every size; by default, calls of about 32 to 18000 cells
+ * staged copies at every size; by default, calls of 17 to some 18000 cells
  * run as one kernel without them, unless the step is so long that many pairs
  * collide, with the same results.)  Applies to later pcc_collide calls on this context; PCC_E_INVALID
  * for polls < 0. */

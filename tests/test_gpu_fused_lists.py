@@ -72,7 +72,7 @@ def run(pcc, wl, fused, graph):
 
 
 @pytest.mark.parametrize("graph", [False, True])
-@pytest.mark.parametrize("law,n_cells", [("many", 40), ("ions", 40), ("edges", 70)])
+@pytest.mark.parametrize("law,n_cells", [("many", 40), ("ions", 40), ("edges", 70), ("many", 17), ("ions", 31)])
 def test_long_lists(pcc, law, n_cells, graph):
     wl = workload(law, n_cells)
     na, st_a, a_stats, a = run(pcc, wl, True, graph)
