@@ -60,18 +60,6 @@ struct WarpGroup {
     __device__ int rank() const { return threadIdx.x & 31; }
     __device__ int size() const { return 32; }
     __device__ void sync() const { __syncwarp(); }
-    template <typename T> __device__ T sum(T v) const { return warp_sum(v); }
-    __device__ float fmin(float v) const
-    {
-        for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        return v;
-    }
-    __device__ float fmax(float v) const
-    {
-        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        return v;
-    }
-    __device__ bool any(bool p) const { return __any_sync(0xffffffffu, p); }
 };
 
 struct CtaGroup {
@@ -89,18 +77,6 @@ struct CtaGroup {
         __syncthreads();
         T t = 0;
         for (int k = 0; k < nw; ++k) t += (T)red[k];
-        return t;
-    }
-    __device__ float fmin(float v) const { return -fmax(-v); }
-    __device__ float fmax(float v) const
-    {
-        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) red[w] = (double)v;
-        __syncthreads();
-        float t = (float)red[0];
-        for (int k = 1; k < nw; ++k) t = fmaxf(t, (float)red[k]);
         return t;
     }
     __device__ bool any(bool p) const { return __syncthreads_or(p) != 0; }
