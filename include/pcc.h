@@ -308,7 +308,7 @@ int pcc_totals(pcc_ctx *ctx, int n_cells, const pcc_species *sp, int is_photon, 
  * the whole device).  Same result as pcc_totals up to the order of the FP64
  * sums; needs no context.  Its scratch is a fixed 96 KiB array in the
  * library's device memory (held by every GPU that loads the library until
- * the process exits), so n_cells is limited to 4,194,304: larger counts
+ * the process exits).  n_cells is limited to 4,194,304: larger counts
  * return PCC_E_CAPACITY without launching anything.  The first call in a
  * CUDA context (normally once per device, with that device current) looks
  * up the array's device address with cudaGetSymbolAddress and caches it per

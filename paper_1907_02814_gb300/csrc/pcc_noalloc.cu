@@ -29,14 +29,15 @@
 
 namespace {
 
-constexpr int kCellsPerBlock = 1024;
-constexpr int kMaxBlocks = 4096;                       // at most 4,194,304 cells
-constexpr int kGridBlocks = 4 * 152;                   // four resident blocks on each SM
-constexpr long long kMaxCells = (long long)kCellsPerBlock * kMaxBlocks;
+constexpr int kMaxBlocks = 4096;                       // entries of the array that pcc.h states
+constexpr int kGridBlocks = 4 * 152;                   // four resident blocks on each SM; the entries in use
+constexpr long long kMaxCells = 4194304;               // the limit that pcc.h states
 
 // Per-block partial sums {sum W, sum W E, sum W |u|}; every block of a call
 // writes its own three entries before the reduction reads them, so nothing
-// has to start at zero.
+// has to start at zero.  The array and the cell limit are the interface's: the
+// slots are shared out to at most kGridBlocks blocks whatever the cells, and a
+// caller that sized its buffers by the limit finds it unchanged.
 static __device__ __align__(256) double g_partial[3 * kMaxBlocks];
 
 std::mutex g_mutex;
