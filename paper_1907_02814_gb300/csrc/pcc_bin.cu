@@ -673,6 +673,15 @@ __global__ void commit_kernel(SpeciesView sp, int n_cells)
     if (c < n_cells) commit_cell(sp, c);
 }
 
+// For more blocks than fit on the SMs at once: overlapping the kernel before gains
+// nothing there, and its two instructions take a block of this kernel as long as its
+// one load (4e6 cells: 17 us with them, 11 without).
+__global__ void commit_many_kernel(SpeciesView sp, int n_cells)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < n_cells) commit_cell(sp, c);
+}
+
 // ---- FP64 totals: slots shared out to the warps, fixed-order partials per block (see pcc_totals.cuh)
 template <bool PHOTON>
 __global__ void __launch_bounds__(256, 4) totals_kernel(const pcc_species sp, int n_cells, double* partial)
@@ -832,7 +841,9 @@ extern "C" int pcc_append_secondaries(pcc_ctx* ctx, int n_cells, pcc_species* sp
         set_error("pcc_append_secondaries: invalid argument");
         return PCC_E_INVALID;
     }
-    launch_pdl(commit_kernel, (n_cells + 255) / 256, 256, 0, (cudaStream_t)stream, view_of(*sp), n_cells);
+    const int blocks = (n_cells + 255) / 256;
+    if (blocks <= 8 * ctx->num_sms) launch_pdl(commit_kernel, blocks, 256, 0, (cudaStream_t)stream, view_of(*sp), n_cells);
+    else commit_many_kernel<<<blocks, 256, 0, (cudaStream_t)stream>>>(view_of(*sp), n_cells);
     note_launches(1);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PCC_OK : cuda_fail(e, "pcc_append_secondaries");
