@@ -2950,16 +2950,16 @@ extern "C" int pcc_set_schedule(pcc_ctx* ctx, int min_blocks_per_sm, int blocks_
 }
 
 // Threads of a plain block.  A block waits on the latency of its cell's phases, so
-// once there are more cells than blocks of 128 threads fit on the SMs (8 on each),
-// twice as many blocks of 64 do better: 16384 cells of 256 electrons 318 against
-// 531 us, of 20 electrons 244 against 454, log-normal ones 402 against 511; 2432
-// cells 87 against 115, 64 against 90 and 93 against 110.  With fewer cells the SMs
-// have room, and a cell is done sooner by 128 threads (64 cells 33 against 36 us,
-// log-normal ones 35 against 42).  Blocks of one warp take 238 us for the first of
-// these, but a large cell holds them up (log-normal ones 548 us).
+// with many cells of like size twice as many blocks of 64 threads do better: 16384
+// cells of 256 electrons 307 against 524 us, of 20 electrons 263 against 491 (blocks
+// of one warp take 238 us for the first of these).  Large cells hold up the smaller
+// blocks, the more so the fewer cells there are beside them: log-normal cells, 64
+// against 128 threads, 16384 at 0.1 fs 694/734, at 1 fs 1896/1585 (3542 before blocks
+// rejected pairs by their digits), but 4096 at 1 fs 1394/864, at 3 fs 1888/1141 (1645
+// before), 2432 at 1 fs 1312/768 (1156 before).  So the line lies at 96 cells per SM.
 static int plain_threads(const pcc_ctx* ctx, int n_cells)
 {
-    return n_cells > 8 * ctx->num_sms ? kPlainThreads / 2 : kPlainThreads;
+    return n_cells > 96 * ctx->num_sms ? kPlainThreads / 2 : kPlainThreads;
 }
 
 int collide_groups(pcc_ctx* ctx, const pcc_cells* cells, pcc_species* em, pcc_species* ep, pcc_species* ph,
