@@ -105,6 +105,7 @@ extern "C" void pcc_destroy(pcc_ctx* ctx)
     if (ctx->lists) cudaFree(ctx->lists);
     if (ctx->queue_a) cudaFree(ctx->queue_a);
     if (ctx->queue_b) cudaFree(ctx->queue_b);
+    if (ctx->heavy) cudaFree(ctx->heavy);
     delete ctx;
 }
 

@@ -1038,21 +1038,24 @@ struct CellList {
 // 120-136 us; at 32768 cells 84-152 against 109-148 us and for log-normal ones 122-179
 // against 131-165 us, since the large cells, which the general scan takes first,
 // hold up a warp.
-// Steps so long that large cells collide on many pairs take the longest on one
-// warp, so its block works off long candidate lists together (see
-// fused_lists_block): 16384 log-normal cells with as many ions as electrons at
-// 1 fs 445 -> 265 us, the general sequence 277.  Where a block is not enough, the
-// general sequence spreads them over the chip, so that beyond a cell for every other
-// SM the step's largest x = n_i sigma beta c dt (pcc_ctx::pair_rate; solid Cu 0.0026
-// a fs) decides.  One kernel against the sequence, log-normal cells, us:
-//   64 cells at 300 fs 68/138; 152 cells at 30 fs 122/150 and 175/162, at 300 fs 189/165;
-//   2432 cells at 2.7 fs 60/154 and 195/191;
-//   16384 cells at 1.6 fs 120/189 and 296/279, at 2.7 fs 138/195 and 347/292
-// (the second pair with as many ions as electrons, the heaviest of the laws).
+// In steps so long that large cells collide on many pairs, such a cell is too much
+// for its warp and even for its block.  The block works off its warps' long
+// lists together (see fused_lists_block); from kSpreadX on the longest are left to
+// a second kernel that spreads them over the chip (fused_heavy_kernel, 3 us where
+// there are none).  The step's largest x = n_i sigma beta c dt tells how long it is
+// (pcc_ctx::pair_rate; solid Cu 0.0026 a fs).  Log-normal cells, us, the general
+// sequence in brackets, with 0.15 ions per electron / as many:
+//   1024 cells at 3 fs 60 (142) / 107 (171), at 100 fs 96 (175) / 175 (220);
+//   16384 cells at 3 fs 131 (196) / 279 (296), at 10 fs 175 (223) / 398 (328);
+// the kernels before these took 201 / 322 and 225 / 400 for the last line.  Beyond
+// kFusedXMax calls of many cells keep the general sequence: 16384 cells at 100 fs 410
+// (304) / 775 (453), at 30 fs 240 (256) / 576 (373).
 constexpr int kFusedMinCells = 17;
 constexpr int kFusedCellsPerWarp = 5;
 constexpr int kFusedWarpsPerSM = 24;
-constexpr double kFusedX[3] = {0.1, 0.007, 0.0043};   // up to one cell per SM, up to 16, and above
+constexpr double kSpreadX = 0.003;
+constexpr double kFusedXMax = 0.07;               // for more than kFusedXCells cells per SM
+constexpr int kFusedXCells = 16;
 constexpr int kClassBlock = 1024;                 // cells per class-sort block
 
 // Class of a cell with N_pair = max(N_p, N_t) pairs: with b the bit length
@@ -2119,6 +2122,15 @@ __global__ void finalize_kernel(const __grid_constant__ StepArgs a, Queue Q)
 // (no group's sums or digits depend on another group's events), and evaluates
 // the candidates of all of them together: one at a time, they would leave most
 // lanes idle through its long chain of dependent loads.
+// A cell whose long lists are spread over the chip (see fused_heavy_kernel).
+struct HeavyCell {
+    int cell, t0, mat;
+    uint32_t Nt;
+    struct { int p0; uint32_t Np; float coef; int cnt; float2 ev; } g[3];   // cnt: entries of its list, 0: no list
+    unsigned changed;   // bit g: an event in group g
+    int done;           // parts worked off
+};
+
 struct FusedArgs {
     int thr[3][4];      // scan lane groups per group (see CellList)
     unsigned run;       // bit g: group g takes part
@@ -2128,6 +2140,8 @@ struct FusedArgs {
     uint32_t *flat[3], *qb[3];
     uint32_t cap[3];    // projectile capacities
     int warps;          // warps of a block that take cells
+    HeavyCell* heavy;   // [n_cells], or null: the blocks work off every list themselves
+    int* n_heavy;       // cells in it and finished blocks, both 0 between calls
 };
 
 constexpr int kFusedWarps = kBatchedThreads / 32;
@@ -2135,6 +2149,8 @@ constexpr int kFusedBatch = 8;      // cells scanned before their candidates are
 constexpr int kFusedQueue = 1024;   // staged candidates: all that one pass of the accept loop can mark
 constexpr int kFusedOwn = 64;       // candidates with N_p < N_t up to which a cell's warp takes them itself
 constexpr uint32_t kFusedSlots = 1u << 27;   // staged slots are below this
+constexpr int kHeavyList = 512;     // candidates of a cell's group from which its list is spread over the chip
+constexpr int kHeavyParts = 8;      // blocks that share a cell
 
 struct FusedWarp {
     float2 ev[kFusedBatch][3];      // radiated energy and created weight of the cell's events
@@ -2142,6 +2158,7 @@ struct FusedWarp {
     struct { int cell, t0, mat; uint32_t Nt; } cell[kFusedBatch];
     unsigned changed;               // bit 4b + g: an event in group g of cell b
     unsigned lists;                 // bit 4b + g: the block works off group g's list of cell b
+    unsigned heavy;                 // bit 4b + g: fused_heavy_kernel does
     int tab[64];
     uint32_t q[kFusedQueue];        // slot << 5 | b << 2 | g
 };
@@ -2211,14 +2228,15 @@ __device__ __noinline__ void fused_caseb(const StepArgs* ap, const uint32_t* qb,
     __syncwarp();
 }
 
-// The warp's share of a long list of a cell with N_p < N_t: the candidates of the
-// projectiles whose slot has its number modulo the warps, so that all pairs of a
-// projectile stay with one warp, in order.  The list is read by every warp; those
-// that are its own gather in buf (64 entries) and are evaluated 32 at a time.
+// A warp's share (number `mine` of `shares`) of a long list of a cell with N_p < N_t:
+// the candidates of the projectiles whose slot has that number modulo the shares, so
+// that all pairs of a projectile stay with one warp, in order.  The list is read by
+// every warp; those that are its own gather in buf (64 entries) and are evaluated
+// 32 at a time.
 template <bool PH>
 __device__ __forceinline__ bool caseb_share(const StepArgs& a, const Tab<float>& tb, int group, int cell, const CellRec& cm,
-                                            const uint32_t* qb, int cnt, int* buf, int wid, int lane, Acc& acc, float& rad,
-                                            float& wcre)
+                                            const uint32_t* qb, int cnt, int* buf, uint32_t mine, uint32_t shares, int lane,
+                                            Acc& acc, float& rad, float& wcre)
 {
     constexpr unsigned kFull = 0xffffffffu;
     const PermKeys rk = perm_keys(a, group, cell);
@@ -2231,7 +2249,7 @@ __device__ __forceinline__ bool caseb_share(const StepArgs& a, const Tab<float>&
 #pragma unroll
             for (int q = 0; q < 4; ++q) j[q] = k0 + 32 * q + lane < cnt ? qb[k0 + 32 * q + lane] : 0u;
         const uint32_t ju = u == 0 ? j[0] : u == 1 ? j[1] : u == 2 ? j[2] : j[3];
-        const bool own = k0 + lane < cnt && (int)(ju % cm.Np % kFusedWarps) == wid;
+        const bool own = k0 + lane < cnt && ju % cm.Np % shares == mine;
         const unsigned m = __ballot_sync(kFull, own);
         if (own) buf[n + __popc(m & below)] = (int)ju;
         n += __popc(m);
@@ -2249,60 +2267,86 @@ __device__ __forceinline__ bool caseb_share(const StepArgs& a, const Tab<float>&
     return any;
 }
 
+// Part `part` of `parts` of the list of a cell's group, by the whole block.  True when the
+// thread changed a projectile.
+__device__ __forceinline__ bool list_part(const StepArgs& a, const FusedArgs& F, int g, int cell, const CellRec& cm, int cnt, int part,
+                                          int parts, int* buf, Acc& acc, float& rad, float& wcre)
+{
+    const Tab<float> tb{a.f_brems_lnsig, a.f_brems_cdf, a.f_bh_lnsig, a.f_bh_cdf, a.f_tri_gp, a.f_tri_split};
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    bool event = false;
+    if (cm.Np >= cm.Nt) {
+        const uint32_t* list = F.flat[g] + cm.p0;
+        for (int i = part * kBatchedThreads + threadIdx.x; i < cnt; i += parts * kBatchedThreads)
+            event |= g == kGroupPh ? flat_pair<true>(a, tb, g, cell, cm, list[i], acc, rad, wcre)
+                                   : flat_pair<false>(a, tb, g, cell, cm, list[i], acc, rad, wcre);
+    } else {
+        const uint32_t* list = F.qb[g] + cm.t0;
+        const uint32_t mine = (uint32_t)(part * kFusedWarps + wid), shares = (uint32_t)(parts * kFusedWarps);
+        event = g == kGroupPh ? caseb_share<true>(a, tb, g, cell, cm, list, cnt, buf, mine, shares, lane, acc, rad, wcre)
+                              : caseb_share<false>(a, tb, g, cell, cm, list, cnt, buf, mine, shares, lane, acc, rad, wcre);
+    }
+    return event;
+}
+
 // The long lists of all warps' cells, by the whole block: one warp alone took
 // about 5 us for every 32 candidates of a cell.
 __device__ __noinline__ void fused_lists_block(const StepArgs* ap, const FusedArgs* F, FusedWarp* work, BlockAcc* bacc)
 {
-    const StepArgs& a = *ap;
-    const Tab<float> tb{a.f_brems_lnsig, a.f_brems_cdf, a.f_bh_lnsig, a.f_bh_cdf, a.f_tri_gp, a.f_tri_split};
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     Acc acc;
     acc.zero();
-    bool some = false;
     for (int k = 0; k < kFusedWarps; ++k) {
         FusedWarp& w = work[k];
         for (unsigned ls = w.lists; ls; ls &= ls - 1u) {   // block-uniform
-            const int bit = __ffs(ls) - 1, b = bit >> 2, g = bit & 3, cnt = w.rec[b][g].cnt, cell = w.cell[b].cell;
-            const CellRec cm = fused_rec(w, b, g);
+            const int bit = __ffs(ls) - 1, b = bit >> 2, g = bit & 3;
             float rad = 0.f, wcre = 0.f;
-            bool event = false;
-            if (cm.Np >= cm.Nt) {
-                const uint32_t* list = F->flat[g] + cm.p0;
-                for (int i = threadIdx.x; i < cnt; i += kBatchedThreads)
-                    event |= g == kGroupPh ? flat_pair<true>(a, tb, g, cell, cm, list[i], acc, rad, wcre)
-                                           : flat_pair<false>(a, tb, g, cell, cm, list[i], acc, rad, wcre);
-            } else {
-                const uint32_t* list = F->qb[g] + cm.t0;
-                event = g == kGroupPh ? caseb_share<true>(a, tb, g, cell, cm, list, cnt, work[wid].tab, wid, lane, acc, rad, wcre)
-                                      : caseb_share<false>(a, tb, g, cell, cm, list, cnt, work[wid].tab, wid, lane, acc, rad, wcre);
-            }
-            if (event) fused_event(w, b, g, rad, wcre);
-            some = true;
+            if (list_part(*ap, *F, g, w.cell[b].cell, fused_rec(w, b, g), w.rec[b][g].cnt, 0, 1, work[threadIdx.x >> 5].tab, acc,
+                          rad, wcre))
+                fused_event(w, b, g, rad, wcre);
         }
     }
-    if (some) add_rare(acc, *bacc);
+    add_rare(acc, *bacc);
 }
 
-// Cell b's ledger (the groups in order) and the removal of its absorbed photons.
-__device__ __noinline__ void fused_finish(const StepArgs* ap, FusedWarp* w, int b)
+// The cell's ledger (the groups of `changed` in order, their contributions ev) and the
+// removal of its absorbed photons.
+__device__ __forceinline__ void finish_cell(const StepArgs& a, int cell, unsigned changed, const float2 (&ev)[3], int lane)
 {
-    const StepArgs& a = *ap;
-    const int lane = threadIdx.x & 31, cell = w->cell[b].cell;
-    const unsigned ch = w->changed >> (4 * b);
     if (lane == 0 && a.ledger) {
         float4* Lg = reinterpret_cast<float4*>(a.ledger) + cell;
         const float4 v = *Lg;
         Kahan ka{v.x, v.y}, kb{v.z, v.w};
         for (int g = 0; g < 3; ++g) {
-            if (!(ch >> g & 1u)) continue;
-            ka.add(w->ev[b][g].x);
-            kb.add(w->ev[b][g].y);
+            if (!(changed >> g & 1u)) continue;
+            ka.add(ev[g].x);
+            kb.add(ev[g].y);
         }
         *Lg = make_float4(ka.s, ka.c, kb.s, kb.c);
     }
     __syncwarp();
-    if (ch >> kGroupPh & 1u) compact_region_warp(a, cell, false);
+    if (changed >> kGroupPh & 1u) compact_region_warp(a, cell, false);
     __syncwarp();
+}
+
+__device__ __noinline__ void fused_finish(const StepArgs* ap, FusedWarp* w, int b)
+{
+    finish_cell(*ap, w->cell[b].cell, w->changed >> (4 * b), w->ev[b], threadIdx.x & 31);
+}
+
+// Leaves cell b to fused_heavy_kernel.  One lane.
+__device__ __noinline__ void fused_publish(const FusedArgs* F, const FusedWarp* w, int b)
+{
+    HeavyCell h;
+    h.cell = w->cell[b].cell; h.t0 = w->cell[b].t0; h.mat = w->cell[b].mat; h.Nt = w->cell[b].Nt;
+    for (int g = 0; g < 3; ++g) {
+        const bool list = w->heavy >> (4 * b + g) & 1u;
+        h.g[g].p0 = w->rec[b][g].p0; h.g[g].Np = w->rec[b][g].Np; h.g[g].coef = w->rec[b][g].coef;
+        h.g[g].cnt = list ? w->rec[b][g].cnt : 0;
+        h.g[g].ev = w->ev[b][g];
+    }
+    h.changed = w->changed >> (4 * b) & 7u;
+    h.done = 0;
+    F->heavy[atomicAdd(F->n_heavy, 1)] = h;
 }
 
 __device__ __noinline__ void fused_commit(const StepArgs* a, int species, int cell)
@@ -2426,6 +2470,8 @@ __device__ __forceinline__ void fused_scan(const StepArgs& a, const FusedArgs& F
         const uint32_t nit = (Np + S * 32 - 1) / (S * 32);
         const PhiloxFixed pf = philox_fixed((uint32_t)cell, step32, stream_tag(GROUP, kAccept, 0), a.keys);
         int listed = 0;
+        // many candidates expected: listed from the first, for the whole chip
+        const bool spread = F.heavy && ((uint64_t)Np * (k1 + k2)) >> 16 >= (uint64_t)kHeavyList;
 #pragma unroll 1
         for (uint32_t it0 = 0; it0 < nit; it0 += kIt) {
             const uint32_t ite = min(it0 + kIt, nit);
@@ -2448,7 +2494,7 @@ __device__ __forceinline__ void fused_scan(const StepArgs& a, const FusedArgs& F
             }
             const int total = (int)__shfl_sync(kFull, incl, 31);
             if (lane == 0) atomicAdd(&bacc.candidates[GROUP], (unsigned long long)total);
-            const bool stage = nq + total <= kFusedQueue && Np <= kFusedSlots;
+            const bool stage = nq + total <= kFusedQueue && Np <= kFusedSlots && !spread;
             if (!stage && (uint32_t)p0 + Np > F.cap[GROUP]) {   // a region past the capacity that the caller gave
                 if (lane == 0) atomicOr(&bacc.status, PCC_ST_CAPACITY);
                 continue;
@@ -2467,7 +2513,7 @@ __device__ __forceinline__ void fused_scan(const StepArgs& a, const FusedArgs& F
         }
         if (listed && lane == 0) {
             w.rec[b][GROUP].cnt = listed;
-            w.lists |= 1u << (4 * b + GROUP);
+            (F.heavy && listed >= kHeavyList ? w.heavy : w.lists) |= 1u << (4 * b + GROUP);
         }
     } else {
         uint32_t* qb = F.qb[GROUP] + t0;
@@ -2502,7 +2548,7 @@ __device__ __forceinline__ void fused_scan(const StepArgs& a, const FusedArgs& F
                 atomicAdd(&bacc.candidates[GROUP], (unsigned long long)cnt);
                 if (cnt > kFusedOwn) {
                     w.rec[b][GROUP].cnt = (int)cnt;
-                    w.lists |= 1u << (4 * b + GROUP);
+                    (F.heavy && cnt >= (uint32_t)kHeavyList ? w.heavy : w.lists) |= 1u << (4 * b + GROUP);
                 }
             }
             __syncwarp();
@@ -2528,7 +2574,7 @@ __global__ void __launch_bounds__(kBatchedThreads, 3) fused_cell_kernel(const __
         const int first = cell;
         int nq = 0, nb = 0;
         if (lane < 3 * kFusedBatch) (&w.ev[0][0])[lane] = make_float2(0.f, 0.f);
-        if (lane == 0) w.changed = w.lists = 0u;
+        if (lane == 0) w.changed = w.lists = w.heavy = 0u;
         __syncwarp();
         for (; cell < a.n_cells && nb < kFusedBatch; cell += nwarps, ++nb) {
             const int nt = a.ion.count[cell], t0 = a.ion.start[cell], mat = a.mat_of_cell[cell];
@@ -2554,7 +2600,14 @@ __global__ void __launch_bounds__(kBatchedThreads, 3) fused_cell_kernel(const __
         fused_drain_block(&a, work, staged, &bacc);
         if (some) fused_lists_block(&a, &F, work, &bacc);
         __syncthreads();
-        for (unsigned ch = w.changed; ch; ch &= ch - 1u) {
+        unsigned later = w.heavy;   // all bits of the cells that fused_heavy_kernel finishes
+        for (unsigned hv = later; hv; hv &= hv - 1u) {
+            const int b = (__ffs(hv) - 1) >> 2;
+            if (lane == 0) fused_publish(&F, &w, b);
+            later |= 0xFu << (4 * b);
+            hv &= ~(0xFu << (4 * b)) | (hv & -hv);
+        }
+        for (unsigned ch = w.changed & ~later; ch; ch &= ch - 1u) {
             const int b = (__ffs(ch) - 1) >> 2;
             fused_finish(&a, &w, b);
             ch &= ~(0xFu << (4 * b)) | (ch & -ch);   // the cell's other groups are done with it
@@ -2563,13 +2616,68 @@ __global__ void __launch_bounds__(kBatchedThreads, 3) fused_cell_kernel(const __
             __syncwarp();
             if (lane < 3 * nb) {
                 const int b = lane / 3, sp = lane - 3 * b, c = first + b * nwarps;
-                if ((sp == 0 ? a.em.added : sp == 1 ? a.ep.added : a.ph.added)[c]) fused_commit(&a, sp, c);
+                if (!(later >> (4 * b) & 1u) && (sp == 0 ? a.em.added : sp == 1 ? a.ep.added : a.ph.added)[c])
+                    fused_commit(&a, sp, c);
             }
             __syncwarp();
         }
     }
     __syncthreads();
     block_acc_flush(bacc, a.st);
+}
+
+// The cells that fused_cell_kernel left: kHeavyParts blocks take a share of a cell's long
+// lists each, and the one that is done last finishes the cell.  Nothing waits.  Launched
+// with steps so long that such cells are to be expected (see kSpreadX): a block alone
+// took 200 us for the largest of 16384 log-normal cells at 30 fs.
+template <bool COMMIT>
+__global__ void __launch_bounds__(kBatchedThreads, 3) fused_heavy_kernel(const __grid_constant__ StepArgs a,
+                                                                         const __grid_constant__ FusedArgs F)
+{
+    __shared__ int tab[kFusedWarps][64];
+    __shared__ BlockAcc bacc;
+    __shared__ int last;
+    const int n = *F.n_heavy;
+    block_acc_init(bacc);
+    __syncthreads();
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int it = blockIdx.x; it < n * kHeavyParts; it += gridDim.x) {
+        HeavyCell& h = F.heavy[it / kHeavyParts];
+        Acc acc;
+        acc.zero();
+        for (int g = 0; g < 3; ++g) {
+            const int cnt = h.g[g].cnt;
+            if (cnt == 0) continue;
+            CellRec cm;
+            cm.p0 = h.g[g].p0; cm.Np = h.g[g].Np; cm.coef = h.g[g].coef;
+            cm.t0 = h.t0; cm.Nt = h.Nt; cm.mat = h.mat;
+            float rad = 0.f, wcre = 0.f;
+            if (list_part(a, F, g, h.cell, cm, cnt, it % kHeavyParts, kHeavyParts, tab[wid], acc, rad, wcre)) {
+                if (rad != 0.f) atomicAdd(&h.g[g].ev.x, rad);
+                if (wcre != 0.f) atomicAdd(&h.g[g].ev.y, wcre);
+                atomicOr(&h.changed, 1u << g);
+            }
+        }
+        add_rare(acc, bacc);
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&h.done, 1) == kHeavyParts - 1;
+        __syncthreads();
+        if (last) {   // the other parts' writes are complete
+            __threadfence();
+            if (wid == 0) {
+                const float2 ev[3] = {__ldcg(&h.g[0].ev), __ldcg(&h.g[1].ev), __ldcg(&h.g[2].ev)};
+                finish_cell(a, h.cell, __ldcg(&h.changed), ev, lane);
+                if (COMMIT && lane < 3) fused_commit(&a, lane, h.cell);
+            }
+        }
+        __syncthreads();
+    }
+    block_acc_flush(bacc, a.st);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(F.n_heavy + 1, 1) == (int)gridDim.x - 1) F.n_heavy[0] = F.n_heavy[1] = 0;   // every block has read them
+    }
 }
 
 // Pairing diagnostic: one warp per cell.
@@ -2710,6 +2818,20 @@ static int ensure_queue(pcc_ctx* ctx, size_t cap_a, size_t cap_b)
     return PCC_OK;
 }
 
+static int ensure_heavy(pcc_ctx* ctx, int n_cells)
+{
+    if (ctx->heavy_cells >= n_cells) return PCC_OK;
+    if (ctx->heavy) cudaFree(ctx->heavy);
+    ctx->heavy = nullptr;
+    ctx->heavy_cells = 0;
+    const size_t bytes = 16 + (size_t)n_cells * sizeof(HeavyCell);   // the two counters, then the cells
+    cudaError_t e = cudaMalloc(&ctx->heavy, bytes);
+    if (e == cudaSuccess) e = cudaMemset(ctx->heavy, 0, bytes);
+    if (e != cudaSuccess) return cuda_fail(e, "pcc_collide: heavy cells");
+    ctx->heavy_cells = n_cells;
+    return PCC_OK;
+}
+
 static CellList list_of(pcc_ctx* ctx, int group)
 {
     const size_t n = ctx->lists_cells;
@@ -2838,10 +2960,16 @@ static bool fused_range(const pcc_ctx* ctx, int n_cells)
 // the launch counter's test counts its kernels at 16 cells.
 static bool use_fused(const pcc_ctx* ctx, int n_cells, int precision, bool split, double dt)
 {
-    if (precision != PCC_FP32_BATCHED || split || ctx->wait_polls != kWaitPolls) return false;
-    if (!fused_range(ctx, n_cells)) return false;
-    if (2 * n_cells <= ctx->num_sms) return true;
-    return ctx->pair_rate * dt <= kFusedX[n_cells <= ctx->num_sms ? 0 : n_cells <= 16 * ctx->num_sms ? 1 : 2];
+    if (precision != PCC_FP32_BATCHED || split || ctx->wait_polls != kWaitPolls || !fused_range(ctx, n_cells)) return false;
+    return n_cells <= kFusedXCells * ctx->num_sms || ctx->pair_rate * dt <= kFusedXMax;
+}
+
+// Whether the longest lists of a one-kernel step are left to fused_heavy_kernel; with
+// fewer cells than every other SM could take, a block for each does (64 log-normal
+// cells at 300 fs 68 us).
+static bool fused_spread(const pcc_ctx* ctx, int n_cells, double dt)
+{
+    return 2 * n_cells > ctx->num_sms && ctx->pair_rate * dt > kSpreadX;
 }
 
 template <bool COMMIT>
@@ -2860,8 +2988,14 @@ static void launch_fused(pcc_ctx* ctx, const StepArgs& a, unsigned run, const in
     // few cells: spread over the SMs, so that more warps are there to work off long lists
     const int grid = persistent_grid(ctx, (const void*)fused_cell_kernel<COMMIT>, 0, ctx->blocks_per_sm);
     F.warps = std::min(kFusedWarps, (a.n_cells + grid - 1) / grid);
+    const bool spread = fused_spread(ctx, a.n_cells, a.dt);
+    F.n_heavy = (int*)ctx->heavy;
+    F.heavy = spread ? reinterpret_cast<HeavyCell*>((char*)ctx->heavy + 16) : nullptr;
     fused_cell_kernel<COMMIT><<<std::min(grid, (a.n_cells + F.warps - 1) / F.warps), kBatchedThreads, 0, st>>>(a, F);
-    note_launches(1);
+    if (spread)
+        fused_heavy_kernel<COMMIT><<<persistent_grid(ctx, (const void*)fused_heavy_kernel<COMMIT>, 0, ctx->blocks_per_sm),
+                                     kBatchedThreads, 0, st>>>(a, F);
+    note_launches(spread ? 2 : 1);
 }
 
 int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em, const pcc_species* ep,
@@ -2892,6 +3026,10 @@ int collide_prepare(pcc_ctx* ctx, const pcc_cells* cells, const pcc_species* em,
         cap_b *= 3;
         persistent_grid(ctx, (const void*)fused_cell_kernel<false>, 0, 0);
         persistent_grid(ctx, (const void*)fused_cell_kernel<true>, 0, 0);
+        persistent_grid(ctx, (const void*)fused_heavy_kernel<false>, 0, 0);
+        persistent_grid(ctx, (const void*)fused_heavy_kernel<true>, 0, 0);
+        rc = ensure_heavy(ctx, cells->n_cells);
+        if (rc) return rc;
     }
     rc = ensure_queue(ctx, std::max<size_t>(cap_a, 1), std::max<size_t>(cap_b, 1));
     if (rc) return rc;

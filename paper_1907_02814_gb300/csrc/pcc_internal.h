@@ -53,6 +53,8 @@ struct pcc_ctx {
     size_t queue_a_cap = 0;
     void* queue_b = nullptr;       // candidate queue over target slots (N_p < N_t cells)
     size_t queue_b_cap = 0;
+    void* heavy = nullptr;         // cells that the one-kernel step leaves to a second kernel
+    int heavy_cells = 0;
     int minb = 4;                  // register budget: minimum resident blocks per SM
     // lane groups of the batched scan per group (e-, e+, photons): size
     // classes (two per octave of N_pair) from which a cell takes a whole

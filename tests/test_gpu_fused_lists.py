@@ -1,7 +1,8 @@
 """The one-kernel step where candidates are many: more than a warp stages in shared
-memory, and long lists in cells with N_p < N_t, which the block works off
-together; few projectiles with many pairs each; and slots beyond what a staged
-candidate can name.  The same bits as the general sequence."""
+memory, and long lists in cells with N_p < N_t, which the block works off together
+or a second kernel spreads over the chip; few projectiles with many pairs each; and
+slots beyond what a staged candidate can name.  The same bits as the general
+sequence."""
 import numpy as np
 import pytest
 
@@ -72,12 +73,15 @@ def run(pcc, wl, fused, graph):
 
 
 @pytest.mark.parametrize("graph", [False, True])
-@pytest.mark.parametrize("law,n_cells", [("many", 40), ("ions", 40), ("edges", 70), ("many", 17), ("ions", 31)])
+@pytest.mark.parametrize("law,n_cells", [("many", 40), ("ions", 40), ("edges", 70), ("many", 17), ("ions", 31),
+                                         ("many", 100), ("ions", 120), ("edges", 900)])
 def test_long_lists(pcc, law, n_cells, graph):
     wl = workload(law, n_cells)
     na, st_a, a_stats, a = run(pcc, wl, True, graph)
     nb, st_b, b_stats, b = run(pcc, wl, False, graph)
-    assert na < nb and st_a == st_b and not st_a & pcc.ST_CAPACITY
+    # beyond a cell for every other SM the long lists are left to a second kernel
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert na == (2 if 2 * n_cells <= sms else 4) + (0 if graph else 6) < nb and st_a == st_b and not st_a & pcc.ST_CAPACITY
     for f in ("pairs", "accepted", "created", "candidates"):
         assert a_stats[f] == b_stats[f], f
     assert min(a_stats["candidates"]) > 1000 and min(a_stats["created"][0], a_stats["created"][4]) > 20
