@@ -796,7 +796,7 @@ __device__ __forceinline__ uint32_t pair_order(const StepArgs& a, int g, int cel
     return plain ? s : ((it / (32 / S) * G + gl) * (32 / S) + it % (32 / S)) * S + s % S;
 }
 
-// Orders the photons appended to a cell (n of them from slot b on) so that the last
+// Orders the photons appended to a cell (n > 1 of them from slot b on) so that the last
 // r, copies of which stay behind when they are moved down by r, do not depend on the
 // order of atomics: in pair_order, e- before e+, which is how they mostly arrive; of
 // long lists the largest ids come last.  All 32 lanes.
@@ -805,7 +805,6 @@ __device__ __noinline__ void order_added(const StepArgs* ap, int cell, int b, in
     constexpr unsigned kFull = 0xffffffffu;
     const SpeciesView& P = ap->ph;
     const int lane = threadIdx.x & 31;
-    if (n < 2) return;
     if (n > 32) { largest_last(P, b, n, r, lane); return; }
     const int sl = b + min(lane, n - 1);
     const uint64_t id = P.pid[sl];
@@ -864,9 +863,11 @@ __device__ void compact_region_warp(const StepArgs& a, int cell, bool plain)
         if (__any_sync(kFull, hole)) break;
     }
     if (c0 >= Np) return;   // nothing removed
-    int removed = 0;
-    for (int i = c0 + lane; i < Np; i += 32) removed += P.w[p0 + i] == 0.f ? 1 : 0;
-    order_added(&a, cell, p0 + Np, n_all - Np, warp_sum(removed), plain);
+    if (n_all - Np > 1) {
+        int removed = 0;
+        for (int i = c0 + lane; i < Np; i += 32) removed += P.w[p0 + i] == 0.f ? 1 : 0;
+        order_added(&a, cell, p0 + Np, n_all - Np, warp_sum(removed), plain);
+    }
     int wr = c0;            // warp-uniform write position
     for (int b = c0; b < n_all; b += 32 * kU) {
         float ux[kU], uy[kU], uz[kU], w[kU], x[kU];
