@@ -673,9 +673,9 @@ __global__ void commit_kernel(SpeciesView sp, int n_cells)
     if (c < n_cells) commit_cell(sp, c);
 }
 
-// For more blocks than fit on the SMs at once: overlapping the kernel before gains
-// nothing there, and its two instructions take a block of this kernel as long as its
-// one load (4e6 cells: 17 us with them, 11 without).
+// For many blocks on an SM: the overlap's two instructions take a block of this kernel
+// as long as its one load, which in the end is more than the overlap gains (4e6 cells,
+// 103 blocks an SM: 17 us with them, 11 without; 2^20 cells, 27 blocks: 5.1 and 5.6).
 __global__ void commit_many_kernel(SpeciesView sp, int n_cells)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -842,7 +842,7 @@ extern "C" int pcc_append_secondaries(pcc_ctx* ctx, int n_cells, pcc_species* sp
         return PCC_E_INVALID;
     }
     const int blocks = (n_cells + 255) / 256;
-    if (blocks <= 8 * ctx->num_sms) launch_pdl(commit_kernel, blocks, 256, 0, (cudaStream_t)stream, view_of(*sp), n_cells);
+    if (blocks <= 40 * ctx->num_sms) launch_pdl(commit_kernel, blocks, 256, 0, (cudaStream_t)stream, view_of(*sp), n_cells);
     else commit_many_kernel<<<blocks, 256, 0, (cudaStream_t)stream>>>(view_of(*sp), n_cells);
     note_launches(1);
     cudaError_t e = cudaGetLastError();
