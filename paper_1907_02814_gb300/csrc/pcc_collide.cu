@@ -812,6 +812,7 @@ __device__ __noinline__ void order_added(const StepArgs* ap, int cell, int b, in
     const uint32_t j = (uint32_t)(id >> 1) & 0xFFFFu;
     uint32_t key = 0;
     for (int g = 0; g < 2; ++g) {
+        if (!__any_sync(kFull, ep == (g == 1))) continue;
         const uint32_t k = pair_order(*ap, g, cell, j, plain, lane);
         if (ep == (g == 1)) key = k;
     }
