@@ -161,7 +161,7 @@ class ClockSampler:
 
 # Sources of the collision kernels: the ncu summaries in profiles/ carry
 # their hash and are used only while it still matches.
-COLLIDE_SOURCES = ("pcc_collide.cu", "pcc_device.cuh", "pcc_internal.h", "pcc_physics.cuh")
+COLLIDE_SOURCES = ("pcc_collide.cu", "pcc_commit.cuh", "pcc_device.cuh", "pcc_internal.h", "pcc_physics.cuh")
 
 
 def source_hash():

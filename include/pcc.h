@@ -260,10 +260,11 @@ int pcc_get_scan_classes(const pcc_ctx *ctx, int group, int *thresholds);
  * a second bounded wait that lets the copy land.  polls = 0 makes every
  * staged launch time out, to test the status path without a hang or a
  * fault.  (A context with its own limit takes the launch sequence with the
- * staged copies at every size; by default, calls of 17 to some 18000 cells
- * run as one kernel, or two where the step is long, without them (more than some
- * 2000 cells not in steps so long that most pairs collide), with the same results.)  Applies to later pcc_collide calls on this context; PCC_E_INVALID
- * for polls < 0. */
+ * staged copies at every size.  By default, calls of 17 to some 18000 cells run
+ * without them, as one kernel, or two where the step is long; more than some 2000
+ * cells in steps so long that many pairs collide take the sequence.  The results
+ * are the same.)  Applies to later pcc_collide calls on this context;
+ * PCC_E_INVALID for polls < 0. */
 int pcc_set_wait_limit(pcc_ctx *ctx, int polls);
 
 /* Make the secondaries of the last step live (Sec. III.A: created

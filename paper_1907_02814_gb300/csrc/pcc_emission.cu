@@ -18,7 +18,7 @@
 // lanes over the nodes, the per-sample factors, the compensated sums and the
 // pair rate cost as much as the nodes, and a lane evaluated exp and expm1 of the
 // same few numbers for every sample.  4096 cells x 512 samples x 64 nodes:
-// forward 2.05 -> 0.52 ms, adjoint 2.91 -> 0.84 ms, bound by FP32 issue.
+// forward 2.05 -> 0.53 ms, adjoint 2.91 -> 0.85 ms, bound by FP32 issue.
 //
 // Precision.  Nodes run in FP32.  The printed closed form of I2 (Eq. deriv_I2)
 // cancels terms of size (L delta)^2 ln L down to O(1), which destroys FP32 once
