@@ -2123,7 +2123,9 @@ __global__ void finalize_kernel(const __grid_constant__ StepArgs a, Queue Q)
 // the same bits on both paths.  A warp scans up to kFusedBatch cells, all groups
 // (no group's sums or digits depend on another group's events), and evaluates
 // the candidates of all of them together: one at a time, they would leave most
-// lanes idle through its long chain of dependent loads.
+// lanes idle through its long chain of dependent loads.  In long steps the lists of
+// the largest cells are left to a second kernel (see kSpreadX).
+
 // A cell whose long lists are spread over the chip (see fused_heavy_kernel).
 struct HeavyCell {
     int cell, t0, mat;
